@@ -44,21 +44,16 @@ INSERT_TRAFFIC = {"bytes_per_op": 227.7, "requests_per_op": 3.545, "digest": "a0
 
 
 def insert_kernel_digest() -> str:
-    """Hash of the insert kernel's source: the device core, the streaming
-    insert's chunk function and kernel with its launch bound, and its
-    launcher."""
+    """Hash of the insert kernel's source: the device core, the warp-run probe
+    loops with their kernel, and its launcher."""
     import hashlib
     import re
     csrc = os.path.join(ROOT, "paper_1908_05936_gb300", "csrc")
     read = lambda f: open(os.path.join(csrc, f)).read()
-    stream, kernels = read("hc_stream.cuh"), read("hc_kernels.cuh")
     parts = [open(os.path.join(ROOT, "include", "hc_core.cuh")).read(),
-             re.search(r"#ifndef HC_STREAM_INSERT_MINB.*?#endif", stream, re.S).group(0),
-             re.search(r"template <class T, int KPT>\nstruct Stage \{.*?\n\};\n", stream, re.S).group(0),
-             re.search(r"__device__ __forceinline__ void insert_stream_chunk\(.*?\n}\n", stream, re.S).group(0),
-             re.search(r"template <int KIND, int BB, int KPT, int S>\n__global__[^\n]*\nk_insert_stream\(.*?\n}\n",
-                       stream, re.S).group(0),
-             re.search(r"cudaError_t launch_insert_stream\(.*?\n}\n", kernels, re.S).group(0)]
+             re.search(r"// -+ warp stacks -+\n.*?\n// Streaming map lookup by lane pairs", read("hc_stream.cuh"),
+                       re.S).group(0),
+             re.search(r"cudaError_t launch_run\(.*?\n}\n", read("hc_kernels.cuh"), re.S).group(0)]
     return hashlib.sha256("\n".join(parts).encode()).hexdigest()[:16]
 
 
@@ -335,7 +330,7 @@ def run_gpu(args, rank: int, world: int):
     achieved = BYTES_PER_OP[kinds[dom]] * dom_n / (dom_ms * 1e-3) / 1e9
     traffic = None
     if (dom == "insert" and not in_kernel and bb == 64 and t.get_launch(0)["keys_per_group"] == 4
-            and t.get_launch(0)["block"] == 64 and insert_kernel_digest() == INSERT_TRAFFIC["digest"]):
+            and t.get_launch(0)["block"] == 128 and insert_kernel_digest() == INSERT_TRAFFIC["digest"]):
         traffic = INSERT_TRAFFIC["bytes_per_op"] * dom_n      # DRAM bytes per launch
     peak, peak_src = hbm_peak()
     ceiling = random_read_ceiling(torch, L)

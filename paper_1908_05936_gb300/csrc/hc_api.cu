@@ -202,15 +202,6 @@ hc_rc run_range(hc_table *t, int op, const void *keys, const void *vals, long lo
     sh.sms = sm_count_of(t->device);
     hc::View v = t->view;
     v.rotate = n > (long long)v.nb ? 1 : 0;        // several inserters per bucket: spread them
-    // Default shape, a plain insert too small to fill the GPU with 4 keys per
-    // thread, into a table larger than L2 with at most one inserter per
-    // bucket: one key per thread in lock step, which keeps more probes in
-    // flight there (measured on a 4 GiB map: +5-12 % for 2^16-2^20 keys).
-    // Crowded or L2-resident inserts and inserts that skip keys keep the
-    // streaming form (an 8 MiB set<u32> took 2.4x as long in lock step).
-    if (op == hc::OP_INSERT && !t->shape_set[op] && !skip && !v.rotate && n < (long long)sh.sms * 8192 &&
-        (long long)v.nb * t->bucket_bytes > l2_bytes_of(t->device))
-        sh.keys_per_group = 1;
     cudaError_t e = dispatch_range(t->kind, op, v, t->bucket_bytes, keys, is_map(t->kind) ? vals : nullptr, n,
                                    out, is_map(t->kind) ? vals_out : nullptr, sh, skip, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the range kernel");
@@ -354,10 +345,8 @@ hc_rc hc_create(hc_table **out, int32_t kind, int64_t slots, const hc_config *cf
         return fail(HC_ERR_OOM, "cudaMalloc of %lld bytes failed: %s", (long long)g.bytes, cudaGetErrorString(e));
     }
     t->view = make_view(t->d_mem, g, seed, hm);
-    // the streaming kernels, one thread per key reading the bucket's keys,
-    // 4 keys per thread with 2 probes in flight, 64-thread blocks: the best
-    // shape of the sweeps on GB300 for uniform keys, for every kind and op.
-    for (int op = 0; op < 3; ++op) t->shape[op] = hc::LaunchShape{key_region_bytes(kind, bb), 4, 64, 0, 0};
+    // the warp-run kernels with runs of up to 128 keys, 128-thread blocks
+    for (int op = 0; op < 3; ++op) t->shape[op] = hc::LaunchShape{key_region_bytes(kind, bb), 4, 128, 0, 0};
     e = dispatch_clear(t, t->view, t->phys, t->capacity, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
         cudaFree(t->d_mem);
@@ -628,8 +617,8 @@ hc_rc hc_erase_ordered(hc_table *t, const void *d_keys, int64_t n, uint8_t *d_st
     const int sms = sm_count_of(t->device);
     cudaError_t e = hc::ordered_leaders(d_keys, key_bytes(t->kind), n, d_scratch, &t->view.hdr->err, sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "finding the first occurrences");
-    // the streaming erase takes the skip flags (later occurrences: NOT_FOUND)
-    hc::LaunchShape sh{key_region_bytes(t->kind, t->bucket_bytes), 4, 64, 0, sms};
+    // the warp-run erase takes the skip flags (later occurrences: NOT_FOUND)
+    hc::LaunchShape sh{key_region_bytes(t->kind, t->bucket_bytes), 4, 128, 0, sms};
     e = dispatch_range(t->kind, hc::OP_ERASE, t->view, t->bucket_bytes, d_keys, nullptr, n, d_status, nullptr, sh,
                        hc::ordered_skip(n, d_scratch), s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the erase kernel");

@@ -89,44 +89,51 @@ k_batch_phase(const BatchItemDev *__restrict__ items, int n_items, long long n_c
     }
 }
 
-// The streaming form of a phase (keys_per_group 4 or 8): a block takes the
-// next chunk with one atomic add and works through it in pieces of
-// blockDim.x * KPT keys with the streaming kernels' chunk functions (keys
-// staged in shared memory, S probes in flight per thread).
-template <int KIND, int OP, int BB, int KPT, int S>
-__global__ void __launch_bounds__(256)
-k_batch_stream(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile,
-               unsigned long long *counter) {
+// The warp-run form of a phase (keys_per_group 4 or 8): a warp takes the next
+// chunk with one atomic add and works through it in runs of up to R keys with
+// the range kernels' probe loops.
+template <int KIND, int OP, int BB, int R>
+__global__ void __launch_bounds__(256, 5)
+k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile,
+            unsigned long long *counter) {
     using T = Traits<KIND>;
-    __shared__ long long s_chunk;
-    const int piece = blockDim.x * KPT;
+    using Key = typename T::Key;
+    using Val = typename T::Val;
+    extern __shared__ __align__(16) unsigned char smem[];
+    WarpRun<KIND, OP, R> &w = reinterpret_cast<WarpRun<KIND, OP, R> *>(smem)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
     while (true) {
-        if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(counter, 1ull);
-        __syncthreads();
-        const long long c = s_chunk;
-        __syncthreads();                                   // s_chunk is written again only after every thread read it
-        if (c >= n_chunks) break;
+        unsigned long long c = 0;
+        if (lane == 0) c = atomicAdd(counter, 1ull);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if ((long long)c >= n_chunks) break;
         int lo = 0, hi = n_items - 1;                      // last item whose chunk_begin <= c
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (items[mid].chunk_begin <= c) lo = mid;
+            if (items[mid].chunk_begin <= (long long)c) lo = mid;
             else hi = mid - 1;
         }
         const BatchItemDev &it = items[lo];
-        const long long k0 = (c - it.chunk_begin) * tile;
+        const View v = it.v;
+        const long long k0 = ((long long)c - it.chunk_begin) * tile;
         const long long k1 = k0 + tile < it.n ? k0 + tile : it.n;
-        const auto *keys = (const typename T::Key *)it.keys;
-        for (long long p0 = k0; p0 < k1; p0 += piece) {
-            const int m = (int)(k1 - p0 < piece ? k1 - p0 : piece);
-            debug_range(it.v, p0, m, it.n);
-            if constexpr (OP == OP_INSERT)
-                insert_stream_chunk<KIND, BB, KPT, S>(it.v, keys, (const typename T::Val *)it.vals, p0, m, it.out,
-                                                      nullptr);
-            else if constexpr (OP == OP_FIND)
-                find_stream_chunk<KIND, BB, KPT, S>(it.v, keys, p0, m, it.out, (typename T::Val *)it.vals_out);
-            else
-                erase_stream_chunk<KIND, BB, KPT, S>(it.v, keys, p0, m, it.out, nullptr);
+        Counts cnts;
+        for (long long p0 = k0; p0 < k1; p0 += R) {
+            const int m = (int)(k1 - p0 < R ? k1 - p0 : R);
+            debug_range(v, p0, m, it.n);
+            ArraySrc<KIND> src{(const Key *)it.keys + p0, (const Val *)it.vals + p0, nullptr};
+            if constexpr (OP == OP_INSERT) insert_run<KIND, BB>(v, src, m, w.stack, w.st, cnts);
+            else if constexpr (OP == OP_FIND) find_run<KIND, BB>(v, src, m, w.stack, w.st, w.vals);
+            else erase_run<KIND, BB>(v, src, m, w.stack, w.st, cnts);
+            for (int i = lane; i < m; i += 32) {
+                if (it.out) st_stream(it.out + p0 + i, w.st[i]);
+                if constexpr (OP == OP_FIND && T::MAP) {
+                    if (it.vals_out) st_stream((Val *)it.vals_out + p0 + i, w.vals[i]);
+                }
+            }
+            __syncwarp();                                  // the results have left before the next run's
         }
+        if constexpr (OP != OP_FIND) flush_counts(v, cnts);
     }
 }
 
@@ -138,18 +145,25 @@ using PhaseKernel = void (*)(const BatchItemDev *, int, long long, int, unsigned
 
 template <int KIND, int OP, int BB>
 PhaseKernel pick_lb_kpt(int lb, int kpt) {
-    if (kpt == 4) return k_batch_stream<KIND, OP, BB, 4, 2>;
-    if (kpt == 8) return k_batch_stream<KIND, OP, BB, 8, 4>;
+    if (kpt == 4) return k_batch_run<KIND, OP, BB, 128>;
+    if (kpt == 8) return k_batch_run<KIND, OP, BB, 256>;
     if (lb == 0) return kpt == 1 ? k_batch_phase<KIND, OP, BB, 1, 1> : k_batch_phase<KIND, OP, BB, 1, 2>;
     return kpt == 1 ? k_batch_phase<KIND, OP, BB, 0, 1> : k_batch_phase<KIND, OP, BB, 0, 2>;
 }
 
-// Dynamic shared memory of a phase launch (the streaming form's staging).
-size_t phase_smem(int kind, int kpt, int block) {
+// Dynamic shared memory of a phase launch (the warp-run form's stacks and results).
+template <int KIND>
+size_t run_smem(int op, int kpt) {
+    if (kpt == 4) return op == OP_INSERT ? sizeof(WarpRun<KIND, 0, 128>) : op == OP_FIND ? sizeof(WarpRun<KIND, 1, 128>) : sizeof(WarpRun<KIND, 2, 128>);
+    return op == OP_INSERT ? sizeof(WarpRun<KIND, 0, 256>) : op == OP_FIND ? sizeof(WarpRun<KIND, 1, 256>) : sizeof(WarpRun<KIND, 2, 256>);
+}
+
+size_t phase_smem(int kind, int op, int kpt, int block) {
     if (kpt < 4) return 0;
-    const int kb = kind == KIND_SET_U32 ? 4 : 8;
-    const int vb = kind == KIND_SET_U32 ? 4 : 8;            // the staging holds a value slot for every kind
-    return stream_smem((long long)block * kpt, kb, vb);
+    const size_t warp = kind == KIND_SET_U32 ? run_smem<KIND_SET_U32>(op, kpt)
+                        : kind == KIND_SET_U64 ? run_smem<KIND_SET_U64>(op, kpt)
+                        : kind == KIND_MAP_I64_I32 ? run_smem<KIND_MAP_I64_I32>(op, kpt) : run_smem<KIND_MAP_U64_U64>(op, kpt);
+    return warp * (size_t)(block / 32);
 }
 
 // A phase kernel with more than the default 48 KB of dynamic shared memory
@@ -239,7 +253,7 @@ hc_rc enqueue(hc_batch *b, cudaStream_t s) {
     for (size_t p = 0; p < b->phases.size(); ++p) {
         const hc::PhaseDesc &ph = b->phases[p];
         hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, b->lane_bytes, b->kpt);
-        const size_t smem = hc::phase_smem(ph.kind, b->kpt, b->block);
+        const size_t smem = hc::phase_smem(ph.kind, ph.op, b->kpt, b->block);
         hc::allow_phase_smem(k, smem);
         k<<<b->grid[p], b->block, smem, s>>>(
             b->d_items + ph.item0, ph.n_items, ph.n_chunks, b->tile, b->d_counters + ph.counter);
@@ -266,7 +280,7 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     const int tile = c.tile ? c.tile : auto_tile(items, n_items);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
-        return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (streaming)");
+        return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
     if (kpt >= 4 && block > 256) return bfail(HC_ERR_ARG, "streaming phases take at most 256 threads per block");
     if (block < 64 || block > 256 || block % 32) return bfail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     if (tile < 128 || tile % 128) return bfail(HC_ERR_ARG, "tile must be a positive multiple of 128");
@@ -337,14 +351,14 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
         int per_sm = c.blocks_per_sm;
         if (per_sm <= 0) {
             hc::PhaseKernel k = hc::pick_kernel(phases[p].kind, phases[p].op, phases[p].bb, lb, kpt);
-            const size_t smem = hc::phase_smem(phases[p].kind, kpt, block);
+            const size_t smem = hc::phase_smem(phases[p].kind, phases[p].op, kpt, block);
             hc::allow_phase_smem(k, smem);
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
             if (per_sm <= 0) per_sm = 1;
         }
         long long g = (long long)sms * per_sm;
-        // one warp (lock-step) or one block (streaming) per chunk at most
-        const long long need = kpt >= 4 ? phases[p].n_chunks : (phases[p].n_chunks * 32 + block - 1) / block;
+        // one warp per chunk at most
+        const long long need = (phases[p].n_chunks * 32 + block - 1) / block;
         if (g > need) g = need;
         b->grid.push_back((int)(g > 0 ? g : 1));
     }
@@ -464,7 +478,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     const int tile = c.tile ? c.tile : auto_tile(items, n_items);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
-        return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (streaming)");
+        return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
     if (kpt >= 4 && block > 256) return bfail(HC_ERR_ARG, "streaming phases take at most 256 threads per block");
     if (block < 64 || block > 256 || block % 32) return bfail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     if (tile < 128 || tile % 128) return bfail(HC_ERR_ARG, "tile must be a positive multiple of 128");
@@ -532,7 +546,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     for (int p = 0; p < n_phases; ++p) {
         const hc::PhaseDesc &ph = phases[p];
         hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lb, kpt);
-        const size_t smem = hc::phase_smem(ph.kind, kpt, block);
+        const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
         hc::allow_phase_smem(k, smem);
         int per_sm = c.blocks_per_sm;
         if (per_sm <= 0) {
@@ -541,7 +555,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
             if (per_sm <= 0) per_sm = 1;
         }
         long long g = (long long)sms * per_sm;
-        const long long need = kpt >= 4 ? ph.n_chunks : (ph.n_chunks * 32 + block - 1) / block;
+        const long long need = (ph.n_chunks * 32 + block - 1) / block;
         if (g > need) g = need;
         k<<<(unsigned)(g > 0 ? g : 1), block, smem, s>>>(
             scratch->items + ph.item0, ph.n_items, ph.n_chunks, tile, scratch->counters + ph.counter);
@@ -603,7 +617,7 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     const int tile = c.tile ? c.tile : auto_tile(items, n_items);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole key region) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
-        return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (streaming)");
+        return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
     if (kpt >= 4 && block > 256) return bfail(HC_ERR_ARG, "streaming phases take at most 256 threads per block");
     if (block < 64 || block > 256 || block % 32) return bfail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     if (tile < 128 || tile % 128) return bfail(HC_ERR_ARG, "tile must be a positive multiple of 128");
@@ -660,12 +674,12 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
         const hc::PhaseDesc &ph = phases[p];
         hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lb, kpt);
         int per_sm = c.blocks_per_sm;
-        const size_t smem = hc::phase_smem(ph.kind, kpt, block);
+        const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
         hc::allow_phase_smem(k, smem);
         if (per_sm <= 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem) != cudaSuccess) per_sm = 1;
         if (per_sm <= 0) per_sm = 1;
         long long g = (long long)sms * per_sm;
-        const long long want = kpt >= 4 ? ph.n_chunks : (ph.n_chunks * 32 + block - 1) / block;
+        const long long want = (ph.n_chunks * 32 + block - 1) / block;
         if (g > want) g = want;
         k<<<(unsigned)(g > 0 ? g : 1), block, smem, s>>>(d_items + ph.item0, ph.n_items, ph.n_chunks, tile,
                                                          d_ctr + ph.counter);

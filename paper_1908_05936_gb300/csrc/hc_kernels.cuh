@@ -184,18 +184,26 @@ void allow_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024) (void)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// Streaming lookup: each thread owns KPT keys of its block's staged chunk and
-// keeps S probes in flight (find only, one thread per key).
-template <int KIND, int BB, int KPT, int S>
-cudaError_t launch_find_stream(const View &v, const void *keys, long long n, uint8_t *out, void *vals_out, int block,
-                               cudaStream_t s) {
+// The warp-run kernels (keys_per_group 4 or 8): runs of up to R = 128 or 256
+// keys per warp, shorter where n is too small to give every SM kRunWarps warps
+// (2^20 keys on a 1 GiB map, runs of 128 against 256: present lookups 19.1 and
+// 17.8 G/s, absent 16.6 and 14.6, inserts 9.5 and 8.4; from 2^24 keys on the
+// two are within 3 %, and runs of 64 gain 2-5 % on lookups and inserts but
+// lose as much on erases).
+constexpr int kRunWarps = 48;
+
+template <int KIND, int BB, int OP, int R>
+cudaError_t launch_run(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
+                       const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     using T = Traits<KIND>;
-    const long long chunk = (long long)block * KPT;
-    const unsigned grid = (unsigned)((n + chunk - 1) / chunk);
-    const size_t smem = stream_smem(chunk, sizeof(typename T::Key), sizeof(typename T::Val));
-    allow_smem(k_find_stream<KIND, BB, KPT, S>, smem);
-    k_find_stream<KIND, BB, KPT, S><<<grid, block, smem, s>>>(v, (const typename T::Key *)keys, n, out,
-                                                              (typename T::Val *)vals_out);
+    const long long even = (n + (long long)sh.sms * kRunWarps - 1) / ((long long)sh.sms * kRunWarps);
+    const int run = (int)std::min<long long>(R, (even + 31) / 32 * 32);
+    const long long per_block = (long long)(sh.block / 32) * run;
+    const unsigned grid = (unsigned)((n + per_block - 1) / per_block);
+    const size_t smem = sizeof(WarpRun<KIND, OP, R>) * (sh.block / 32);
+    allow_smem(k_run<KIND, BB, OP, R>, smem);
+    k_run<KIND, BB, OP, R><<<grid, sh.block, smem, s>>>(v, (const typename T::Key *)keys, (const typename T::Val *)vals,
+                                                        skip, n, run, out, (typename T::Val *)vals_out);
     return cudaGetLastError();
 }
 
@@ -208,31 +216,6 @@ cudaError_t launch_find_pair(const View &v, const void *keys, long long n, uint8
     const size_t smem = (size_t)chunk * (sizeof(typename T::Key) + sizeof(typename T::Val) + 1);
     k_find_pair<KIND, BB, KPT, S><<<grid, block, smem, s>>>(v, (const typename T::Key *)keys, n, out,
                                                             (typename T::Val *)vals_out);
-    return cudaGetLastError();
-}
-
-template <int KIND, int BB, int KPT, int S>
-cudaError_t launch_insert_stream(const View &v, const void *keys, const void *vals, long long n, uint8_t *out,
-                                 const uint8_t *skip, int block, cudaStream_t s) {
-    using T = Traits<KIND>;
-    const long long chunk = (long long)block * KPT;
-    const unsigned grid = (unsigned)((n + chunk - 1) / chunk);
-    const size_t smem = stream_smem(chunk, sizeof(typename T::Key), sizeof(typename T::Val));
-    allow_smem(k_insert_stream<KIND, BB, KPT, S>, smem);
-    k_insert_stream<KIND, BB, KPT, S><<<grid, block, smem, s>>>(v, (const typename T::Key *)keys,
-                                                                (const typename T::Val *)vals, n, out, skip);
-    return cudaGetLastError();
-}
-
-template <int KIND, int BB, int KPT, int S>
-cudaError_t launch_erase_stream(const View &v, const void *keys, long long n, uint8_t *out, const uint8_t *skip,
-                                int block, cudaStream_t s) {
-    using T = Traits<KIND>;
-    const long long chunk = (long long)block * KPT;
-    const unsigned grid = (unsigned)((n + chunk - 1) / chunk);
-    const size_t smem = stream_smem(chunk, sizeof(typename T::Key), 0);
-    allow_smem(k_erase_stream<KIND, BB, KPT, S>, smem);
-    k_erase_stream<KIND, BB, KPT, S><<<grid, block, smem, s>>>(v, (const typename T::Key *)keys, n, out, skip);
     return cudaGetLastError();
 }
 
@@ -250,16 +233,16 @@ cudaError_t launch_range_kpt(int op, const View &v, const void *keys, const void
         }
         if constexpr (LB == Slots<KIND, BB>::KRB) {
             if (n <= 0) return cudaSuccess;
-            if (op == OP_FIND) {
-                if (sh.keys_per_group == 4) return launch_find_stream<KIND, BB, 4, 2>(v, keys, n, out, vals_out, sh.block, s);
-                if (sh.keys_per_group == 8) return launch_find_stream<KIND, BB, 8, 4>(v, keys, n, out, vals_out, sh.block, s);
-            } else if (op == OP_INSERT) {
-                if (sh.keys_per_group == 4) return launch_insert_stream<KIND, BB, 4, 2>(v, keys, vals, n, out, skip, sh.block, s);
-                if (sh.keys_per_group == 8) return launch_insert_stream<KIND, BB, 8, 4>(v, keys, vals, n, out, skip, sh.block, s);
-            } else {
-                if (sh.keys_per_group == 4) return launch_erase_stream<KIND, BB, 4, 2>(v, keys, n, out, skip, sh.block, s);
-                if (sh.keys_per_group == 8) return launch_erase_stream<KIND, BB, 8, 4>(v, keys, n, out, skip, sh.block, s);
-            }
+            const bool small = sh.keys_per_group == 4;
+            if (!small && sh.keys_per_group != 8) return cudaErrorInvalidValue;
+            if (op == OP_INSERT)
+                return small ? launch_run<KIND, BB, OP_INSERT, 128>(v, keys, vals, n, out, nullptr, sh, skip, s)
+                             : launch_run<KIND, BB, OP_INSERT, 256>(v, keys, vals, n, out, nullptr, sh, skip, s);
+            if (op == OP_FIND)
+                return small ? launch_run<KIND, BB, OP_FIND, 128>(v, keys, nullptr, n, out, vals_out, sh, nullptr, s)
+                             : launch_run<KIND, BB, OP_FIND, 256>(v, keys, nullptr, n, out, vals_out, sh, nullptr, s);
+            return small ? launch_run<KIND, BB, OP_ERASE, 128>(v, keys, nullptr, n, out, nullptr, sh, skip, s)
+                         : launch_run<KIND, BB, OP_ERASE, 256>(v, keys, nullptr, n, out, nullptr, sh, skip, s);
         }
         return cudaErrorInvalidValue;
     }

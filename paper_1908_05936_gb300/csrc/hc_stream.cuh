@@ -1,27 +1,8 @@
-// hc_stream.cuh -- the streaming range kernels: a block stages its chunk of
-// keys (and values) in shared memory with coalesced 16-byte loads, so the key
-// load leaves each key's chain of dependent reads.  Every thread then keeps S
-// probes in flight and refills a slot from the chunk as soon as its probe
-// finishes (instead of moving its keys in lock-step rounds); a key is hashed
-// when its slot takes it, while the other slots' reads are in flight.
-// Results go to shared memory and leave in coalesced stores.  One thread per
-// key, reading the bucket's key region (KRB bytes) per probe.
+// hc_stream.cuh -- the default range kernels (warp runs), shared by the
+// batched form, and the lane-pair lookup.
 #pragma once
 
 #include "hc_core.cuh"
-
-// Minimum resident 256-thread blocks per SM requested from the compiler
-// (__launch_bounds__), i.e. a register cap of 65536 / (256 * MINB) per
-// thread; build options.
-#ifndef HC_STREAM_FIND_MINB
-#define HC_STREAM_FIND_MINB 1
-#endif
-#ifndef HC_STREAM_INSERT_MINB
-#define HC_STREAM_INSERT_MINB 1
-#endif
-#ifndef HC_STREAM_ERASE_MINB
-#define HC_STREAM_ERASE_MINB 1
-#endif
 
 // Lookups read buckets through L1 (the read-only path) when 1: a lookup
 // never runs together with a modifying call on its table, so the line a
@@ -103,12 +84,6 @@ struct Stage {
     }
 };
 
-// Dynamic shared memory of the streaming kernels for a chunk of `chunk`
-// keys: per key its key, value (vb bytes; 0 for erase) and result byte.
-__host__ __device__ __forceinline__ size_t stream_smem(long long chunk, int kb, int vb) {
-    return (size_t)chunk * (kb + vb + 1);
-}
-
 template <int LB>
 __device__ __forceinline__ void load_find(LaneWords<LB> &lw, const unsigned char *p) {
     if constexpr (HC_FIND_L1 && LB >= 32) {
@@ -131,108 +106,703 @@ __device__ __forceinline__ unsigned long long load_find_val(const View &v, unsig
         return load_val<KIND, BB>(v, b, s);
 }
 
-template <int KIND, int BB, int KPT, int S>
-__device__ __forceinline__ void find_stream_chunk(const View &v, const typename Traits<KIND>::Key *keys, long long c0, int m,
-                                                  uint8_t *found, typename Traits<KIND>::Val *vals_out) {
+// ---------------------------------------------------------- warp stacks ---
+// The probe loops of the range kernels.  A warp works through a run of keys in
+// steps; in a step every lane reads one bucket for one key.  Keys that stay
+// undecided go onto the warp's stack in shared memory, and a step takes 32 of
+// them as soon as there are that many, the next 32 keys of the run otherwise.
+// So all lanes of a step do the same thing on a key of their own until the run
+// ends, and the state of a key in flight is one stack entry (about 40-50
+// registers a thread against 64-128 with two whole probes in registers).
+//
+// What bounds it: beyond L2, the device's scattered requests (about 50 G/s on
+// a 4 GiB table); inside L2, latency and, with a loop in which every lane
+// refills its own probe as soon as it ends, instructions: such a loop runs its
+// whole body, hashing included, for the few lanes at each point of it.
+// Against that loop (keys staged per block, two probes in flight per thread):
+// a pass over 400,000 RGB-D candidates (lookup, insert, lookup, erase; spatial
+// hash, 12.5 M slots) 129 -> 72 us; 10^6 inserts + lookups + erases on a
+// 50 M-slot map at load factor 0.7, 331 -> 236 us; 2^26 lookups, half of them
+// present, on 2^28 slots at 0.8, 4.21 -> 3.56 ms; 30 M set lookups on 10^8
+// slots, 0.93 -> 0.84 ms; a 4097-key lookup, call included, 25 -> 17 us.
+constexpr int kStack = 64;           // entries: below 32 left by a step, 32 more pushed by it
+
+__device__ __forceinline__ unsigned lanes_below() {
+    unsigned m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// Whether bucket `next`, the one after the bucket a key has just read, is the
+// key's first bucket again: only then have all nb buckets been read.  A key is
+// at most `reach` buckets from home, so there is nothing to compute before.
+__device__ __forceinline__ bool came_round(const View &v, unsigned long long key, unsigned long long next,
+                                           unsigned long long reach) {
+    return reach + 1 >= v.nb && next == first_bucket(v, key);
+}
+
+// The end of a run, when at most 16 keys are left: G = 32 / 16, 8, 4, 2 or 1
+// lanes share a key and read its next G buckets at once, so that the last long
+// probe sequences of a run take a few steps instead of one per bucket.
+// Neighbouring buckets share lines, which a warp's load asks for once.
+// (2^20 inserts into 2^22 L2-resident slots, load factor 0.6 -> 0.85: 7.7 G/s
+// without, 13.5 G/s with; 2^24 absent lookups on 2^28 slots at 0.75: 17.9 and
+// 20.4 G/s.)
+struct Drain {
+    int group;               // lanes per key
+    int entry, sub;          // this lane's stack entry and its bucket after the entry's
+    unsigned base;           // first lane of the group
+    __device__ __forceinline__ explicit Drain(int top) {
+        const int lg = top > 8 ? 1 : top > 4 ? 2 : top > 2 ? 3 : top > 1 ? 4 : 5;
+        const int lane = threadIdx.x & 31;
+        group = 1 << lg;
+        entry = lane >> lg;
+        sub = lane & (group - 1);
+        base = (unsigned)(lane & ~(group - 1));
+    }
+    // bits [0, group) = pred of the group's lanes; the whole warp calls it
+    __device__ __forceinline__ unsigned ballot(bool pred) const {
+        const unsigned m = __ballot_sync(0xffffffffu, pred) >> base;
+        return group == 32 ? m : m & ((1u << group) - 1u);
+    }
+    // Buckets that a key at bucket b has not read yet (up to `group` of them;
+    // exact only when it can have come round).
+    __device__ __forceinline__ int unread(const View &v, unsigned long long key, unsigned long long b,
+                                          unsigned long long reach) const {
+        if (reach + group < v.nb) return group;
+        const unsigned long long home = first_bucket(v, key);
+        const unsigned long long rest = home > b ? home - b : home + v.nb - b;
+        return rest < (unsigned long long)group ? (int)rest : group;
+    }
+    __device__ __forceinline__ static unsigned long long bucket(const View &v, unsigned long long b, int ahead) {
+        b += ahead;
+        return b >= v.nb ? b - v.nb : b;
+    }
+};
+
+// Stack entries: the key, its next bucket << 16 | its position in the run, and
+// for inserts the value and the first free slot the key has passed (slot
+// position << 1 | was EMPTY; all ones: none).
+template <int KIND, int OP>
+struct Stack {
+    using Key = typename Traits<KIND>::Key;
+    using Val = typename Traits<KIND>::Val;
+    static constexpr bool INS = OP == 0, VAL = INS && Traits<KIND>::MAP;
+    unsigned long long at[kStack];
+    unsigned long long free_at[INS ? kStack : 1];
+    Key key[kStack];
+    Val val[VAL ? kStack : 1];
+};
+
+// Looks up the keys src.key(i), i < cnt (asked for 32 at a time, in order, by
+// the whole warp); found flags go to sf[i], values to sv[i].
+template <int KIND, int BB, class Src>
+__device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack<KIND, 1> &st, uint8_t *sf,
+                                         typename Traits<KIND>::Val *sv) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
     using Sl = Slots<KIND, BB>;
     constexpr int LB = Sl::KRB;              // one thread reads the whole key region
-    constexpr int SPL = Sl::SPB;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int nt = blockDim.x;
-    const int chunk = nt * KPT;
-    Key *sk = reinterpret_cast<Key *>(smem);
-    Val *sv = reinterpret_cast<Val *>(smem + (size_t)chunk * sizeof(Key));
-    uint8_t *sf = smem + (size_t)chunk * (sizeof(Key) + sizeof(Val));
-
-    Stage<Key, KPT> gk;
-    gk.load(keys + c0, m);
-    __syncthreads();                         // the staging of a previous chunk is no longer read
-    gk.store(sk, m);
-    __syncthreads();
-
-    // this thread's keys: threadIdx.x + j * nt, j < KPT
-    int idx[S];
-    Key key[S];
-    unsigned long long b[S];
-    uint32_t probes[S];
-    int next = 0;
-    uint32_t active = 0;
-    auto take = [&](int s) {
-        while (next < KPT) {
-            const int i = threadIdx.x + (next++) * nt;
-            if (i >= m) { next = KPT; break; }
-            const Key k = sk[i];
-            const int side = side_index<KIND>(k);
-            if (side >= 0) {
+    const int lane = threadIdx.x & 31;
+    int next = 0, top = 0;
+    Key ahead = lane < cnt ? src.key(lane) : Key();
+    int late = -1;                           // a found key whose value is still on its way
+    Val late_val = Val();
+    unsigned long long reach = 0;
+    const int few = v.nb >= 32 ? 16 : 0;     // a group's buckets are distinct
+    for (;; ++reach) {
+        Key key;
+        unsigned long long b = 0;
+        int idx;
+        bool act;
+        if (top < 32 && next < cnt) {
+            key = ahead;
+            idx = next + lane;
+            act = idx < cnt;
+            next += 32;
+            if (next + lane < cnt) ahead = src.key(next + lane);
+            const int side = side_index<KIND>(key);
+            if (act && side >= 0) {          // key equal to a marker: side slot
                 const uint32_t pres = *((volatile unsigned int *)&v.hdr->side_present[side]);
-                sf[i] = pres ? 1 : 0;
-                if constexpr (T::MAP) sv[i] = pres ? (Val) * ((volatile unsigned long long *)&v.hdr->side_val[side]) : (Val)0;
-                continue;
+                sf[idx] = pres ? 1 : 0;
+                if constexpr (T::MAP)
+                    sv[idx] = pres ? (Val) * ((volatile unsigned long long *)&v.hdr->side_val[side]) : (Val)0;
+                act = false;
             }
-            idx[s] = i;
-            key[s] = k;
-            b[s] = first_bucket(v, (unsigned long long)k);
-            probes[s] = 0;
-            active |= 1u << s;
-            return;
+            b = first_bucket(v, (unsigned long long)key);
+        } else if (top > few) {
+            const int take = top < 32 ? top : 32;
+            top -= take;
+            act = lane < take;
+            const unsigned long long e = st.at[top + (act ? lane : 0)];
+            key = st.key[top + (act ? lane : 0)];
+            idx = (int)(e & 0xffffu);
+            b = e >> 16;
+        } else {
+            break;
         }
-    };
-#pragma unroll
-    for (int s = 0; s < S; ++s) take(s);
-    while (active) {
-        LaneWords<LB> lw[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-            if (active >> s & 1u) load_find<LB>(lw[s], bucket_at<BB>(v, b[s]));
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(active >> s & 1u)) continue;
-            uint32_t lm = 0, le = 0;
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                const Key ks = slot_key<KIND, LB>(lw[s], q);
-                lm |= (uint32_t)(ks == key[s]) << q;
-                le |= (uint32_t)(ks == T::EMPTY) << q;
-            }
-            bool done = false;
-            if (lm) {
-                sf[idx[s]] = 1;
-                if constexpr (T::MAP) sv[idx[s]] = (Val)load_find_val<KIND, BB>(v, b[s], __ffs(lm) - 1);
-                done = true;
-            } else if (le || ++probes[s] >= v.nb) {
-                sf[idx[s]] = 0;
-                if constexpr (T::MAP) sv[idx[s]] = (Val)0;
-                done = true;
-            } else {
-                b[s] = next_bucket(v, b[s]);
-            }
-            if (done) {
-                active &= ~(1u << s);
-                take(s);
-            }
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += nt) {
-        if (found) st_stream(found + c0 + i, sf[i]);
+        __syncwarp();                        // entries are read before this step's survivors overwrite them
+        LaneWords<LB> lw;
+        if (act) load_find<LB>(lw, bucket_at<BB>(v, b));
         if constexpr (T::MAP) {
-            if (vals_out) st_stream(vals_out + c0 + i, sv[i]);
+            if (late >= 0) sv[late] = late_val;
+            late = -1;
         }
+        bool left = false;
+        if (act) {
+            int hit = -1;
+            bool empty = false;
+#pragma unroll
+            for (int x = 0; x < Sl::SPB; ++x) {
+                const Key ks = slot_key<KIND, LB>(lw, x);
+                if (ks == key) hit = x;
+                empty |= ks == T::EMPTY;
+            }
+            if (hit >= 0) {
+                sf[idx] = 1;
+                if constexpr (T::MAP) {
+                    late = idx;
+                    late_val = (Val)load_find_val<KIND, BB>(v, b, hit);
+                }
+            } else {
+                b = next_bucket(v, b);
+                left = !empty && !came_round(v, (unsigned long long)key, b, reach);
+                if (!left) {
+                    sf[idx] = 0;
+                    if constexpr (T::MAP) sv[idx] = (Val)0;
+                }
+            }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int p = top + __popc(mask & lanes_below());
+            st.at[p] = b << 16 | (unsigned)idx;
+            st.key[p] = key;
+        }
+        top += __popc(mask);
+        __syncwarp();
     }
+    if constexpr (T::MAP) {
+        if (late >= 0) sv[late] = late_val;
+    }
+    while (top > 0) {
+        const Drain d(top);
+        const bool act = d.entry < top;
+        const int p = act ? d.entry : 0;
+        const unsigned long long e = st.at[p];
+        const Key key = st.key[p];
+        const int idx = (int)(e & 0xffffu);
+        unsigned long long b = e >> 16;
+        __syncwarp();
+        const int unread = d.unread(v, (unsigned long long)key, b, reach);
+        const unsigned long long mine = Drain::bucket(v, b, d.sub);
+        int hit = -1;
+        bool empty = false;
+        if (act && d.sub < unread) {
+            LaneWords<LB> lw;
+            load_find<LB>(lw, bucket_at<BB>(v, mine));
+#pragma unroll
+            for (int x = 0; x < Sl::SPB; ++x) {
+                const Key ks = slot_key<KIND, LB>(lw, x);
+                if (ks == key) hit = x;
+                empty |= ks == T::EMPTY;
+            }
+        }
+        const unsigned stop = d.ballot(hit >= 0 || empty);
+        bool left = false;
+        if (act && stop) {
+            if (d.sub == __ffs(stop) - 1) {
+                sf[idx] = hit >= 0 ? 1 : 0;
+                if constexpr (T::MAP) sv[idx] = hit >= 0 ? (Val)load_find_val<KIND, BB>(v, mine, hit) : (Val)0;
+            }
+        } else if (act && d.sub == 0) {
+            left = unread == d.group;
+            b = Drain::bucket(v, b, d.group);
+            left = left && !(reach + d.group >= v.nb && b == first_bucket(v, (unsigned long long)key));
+            if (!left) {
+                sf[idx] = 0;
+                if constexpr (T::MAP) sv[idx] = (Val)0;
+            }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int q = __popc(mask & lanes_below());
+            st.at[q] = b << 16 | (unsigned)idx;
+            st.key[q] = key;
+        }
+        top = __popc(mask);
+        reach += d.group;
+        __syncwarp();
+    }
+    __syncwarp();
 }
 
-template <int KIND, int BB, int KPT, int S>
-__global__ void __launch_bounds__(256, HC_STREAM_FIND_MINB)
-k_find_stream(View v, const typename Traits<KIND>::Key *keys, long long n, uint8_t *found,
-              typename Traits<KIND>::Val *vals_out) {
-    const long long chunk = (long long)blockDim.x * KPT;
-    const long long c0 = (long long)blockIdx.x * chunk;
-    const int m = (int)(n - c0 < chunk ? n - c0 : chunk);
-    debug_range(v, c0, m, n);
-    find_stream_chunk<KIND, BB, KPT, S>(v, keys, c0, m, found, vals_out);
+// Inserts the keys src.key(i) with values src.val(i), i < cnt, except those
+// with src.skip(i) (a find saw them: EXISTS); statuses go to ss[i].  A key that
+// loses its slot to another key goes on from that slot's bucket: the buckets
+// before it had no free slot, and inserts never free one.  Equal keys inside a
+// warp are not folded here (folding is a lock-step option).
+template <int KIND, int BB, class Src>
+__device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Stack<KIND, 0> &st, uint8_t *ss,
+                                           Counts &cnts) {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using Val = typename T::Val;
+    using Sl = Slots<KIND, BB>;
+    using Lay = Layout<KIND, BB, Sl::KRB>;
+    constexpr int LB = Sl::KRB;
+    constexpr int SPL = Sl::SPB;
+    constexpr unsigned long long NONE = ~0ull;
+    const int lane = threadIdx.x & 31;
+    int next = 0, top = 0;
+    Key ahead = Key();
+    Val ahead_val = Val();
+    bool ahead_skip = false;
+    auto fetch = [&](int i) {
+        if (i >= cnt) return;
+        ahead = src.key(i);
+        if constexpr (T::MAP) ahead_val = src.val(i);
+        ahead_skip = src.skip(i);
+    };
+    fetch(lane);
+    unsigned long long reach = 0;
+    const int few = v.nb >= 32 ? 16 : 0;     // a group's buckets are distinct
+    // Claims the free slot `at` for key; whether the key stays undecided, with
+    // its next bucket in b (it lost the slot to another key).
+    auto claim_slot = [&](unsigned long long &at, Key key, Val val, int idx, unsigned long long &b) -> bool {
+        const bool was_empty = at & 1;
+        const unsigned long long fb = (at >> 1) / SPL;
+        const int x = (int)((at >> 1) % SPL);
+        const Key expect = was_empty ? T::EMPTY : T::TOMB;
+        const Key old = cas_key<KIND>(Sl::key(v, fb, x), expect, key);
+        if (old == expect) {
+            if constexpr (T::MAP) {
+                store_val<KIND, BB>(v, fb, x, (unsigned long long)val);
+                note_claim_key<KIND>(v.hdr, key, (long long)(at >> 1));
+            }
+            ss[idx] = (uint8_t)ST_INSERTED;
+            ++cnts.ins;
+            cnts.new_slot += was_empty ? 1u : 0u;
+            return false;
+        }
+        if (old == key) {                                    // an equal key won the race
+            ss[idx] = (uint8_t)ST_EXISTS;
+            return false;
+        }
+        if (reach >= v.nb + 32ull * kMaxRestarts) {
+            atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
+            ss[idx] = (uint8_t)ST_OVERFLOW;
+            cnts.over = 1;
+            return false;
+        }
+        b = fb;
+        at = NONE;
+        return true;
+    };
+    for (;; ++reach) {
+        Key key;
+        Val val = Val();
+        unsigned long long b = 0, at = NONE;
+        int idx;
+        bool act;
+        if (top < 32 && next < cnt) {
+            key = ahead;
+            val = ahead_val;
+            idx = next + lane;
+            act = idx < cnt;
+            if (act && ahead_skip) {
+                ss[idx] = (uint8_t)ST_EXISTS;
+                act = false;
+            }
+            next += 32;
+            fetch(next + lane);
+            const int side = side_index<KIND>(key);
+            if (act && side >= 0) {          // key equal to a marker: side slot
+                const bool won = atomicCAS(&v.hdr->side_present[side], 0u, 1u) == 0u;
+                if (won) {
+                    if constexpr (T::MAP) v.hdr->side_val[side] = (unsigned long long)val;
+                    ++cnts.ins;
+                }
+                ss[idx] = won ? (uint8_t)ST_INSERTED : (uint8_t)ST_EXISTS;
+                act = false;
+            }
+            b = first_bucket(v, (unsigned long long)key);
+        } else if (top > few) {
+            const int take = top < 32 ? top : 32;
+            top -= take;
+            act = lane < take;
+            const int p = top + (act ? lane : 0);
+            const unsigned long long e = st.at[p];
+            key = st.key[p];
+            if constexpr (T::MAP) val = st.val[p];
+            at = st.free_at[p];
+            idx = (int)(e & 0xffffu);
+            b = e >> 16;
+        } else {
+            break;
+        }
+        __syncwarp();                        // entries are read before this step's survivors overwrite them
+        LaneWords<LB> lw;
+        if (act) lw.load(bucket_at<BB>(v, b));
+        bool left = false, claim = false;
+        if (act) {
+            bool hit = false;
+            uint32_t le = 0, lt = 0;
+#pragma unroll
+            for (int x = 0; x < SPL; ++x) {
+                const Key ks = slot_key<KIND, LB>(lw, x);
+                hit |= ks == key;
+                le |= (uint32_t)(ks == T::EMPTY) << x;
+                lt |= (uint32_t)(ks == T::TOMB) << x;
+            }
+            if (hit) {                       // already stored
+                ss[idx] = (uint8_t)ST_EXISTS;
+            } else {
+                if (at == NONE) {            // first free slot, rotated scan
+                    const uint32_t lf = le | (lt & claimable<KIND, BB, LB>(v, b, 0));
+                    if (lf) {
+                        const int rot = v.rotate ? slot_rotation<Lay::SPB>((unsigned long long)key) : 0;
+                        const uint32_t hi = lf & (Lay::ALL & ~((1u << rot) - 1u));
+                        const int x = __ffs(hi ? hi : lf) - 1;
+                        at = (b * SPL + x) << 1 | (le >> x & 1u);
+                    }
+                }
+                claim = le != 0;
+                if (!claim) {
+                    b = next_bucket(v, b);
+                    left = !came_round(v, (unsigned long long)key, b, reach);
+                    claim = !left && at != NONE;             // only tombstones were free
+                    if (!left && !claim) {                   // no free slot anywhere
+                        ss[idx] = (uint8_t)ST_OVERFLOW;
+                        cnts.over = 1;
+                    }
+                }
+            }
+        }
+        if (claim) left = claim_slot(at, key, val, idx, b);
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int p = top + __popc(mask & lanes_below());
+            st.at[p] = b << 16 | (unsigned)idx;
+            st.free_at[p] = at;
+            st.key[p] = key;
+            if constexpr (T::MAP) st.val[p] = val;
+        }
+        top += __popc(mask);
+        __syncwarp();
+    }
+    while (top > 0) {
+        const Drain d(top);
+        const bool act = d.entry < top;
+        const int p = act ? d.entry : 0;
+        const unsigned long long e = st.at[p];
+        const Key key = st.key[p];
+        Val val = Val();
+        if constexpr (T::MAP) val = st.val[p];
+        unsigned long long at = st.free_at[p];
+        const int idx = (int)(e & 0xffffu);
+        unsigned long long b = e >> 16;
+        __syncwarp();
+        const int unread = d.unread(v, (unsigned long long)key, b, reach);
+        const unsigned long long mine = Drain::bucket(v, b, d.sub);
+        bool hit = false;
+        uint32_t le = 0;
+        unsigned long long here = NONE;                      // first free slot of this lane's bucket
+        if (act && d.sub < unread) {
+            LaneWords<LB> lw;
+            lw.load(bucket_at<BB>(v, mine));
+            uint32_t lt = 0;
+#pragma unroll
+            for (int x = 0; x < SPL; ++x) {
+                const Key ks = slot_key<KIND, LB>(lw, x);
+                hit |= ks == key;
+                le |= (uint32_t)(ks == T::EMPTY) << x;
+                lt |= (uint32_t)(ks == T::TOMB) << x;
+            }
+            const uint32_t lf = le | (lt & claimable<KIND, BB, LB>(v, mine, 0));
+            if (lf) {
+                const int rot = v.rotate ? slot_rotation<Lay::SPB>((unsigned long long)key) : 0;
+                const uint32_t hi = lf & (Lay::ALL & ~((1u << rot) - 1u));
+                const int x = __ffs(hi ? hi : lf) - 1;
+                here = (mine * SPL + x) << 1 | (le >> x & 1u);
+            }
+        }
+        const unsigned stop = d.ballot(hit || le != 0);
+        const unsigned stored = d.ballot(hit);
+        const unsigned some = d.ballot(here != NONE);
+        const unsigned first = stop & (0u - stop);           // the bucket that ends the probe, if any
+        const unsigned upto = first ? (first - 1u) | first : 0xffffffffu;
+        const unsigned from = some & upto;                   // free slots the probe passes
+        const unsigned long long passed =
+            __shfl_sync(0xffffffffu, here, (int)d.base + (from ? __ffs(from) - 1 : 0));
+        bool left = false;
+        if (act && d.sub == 0) {
+            if (at == NONE && from) at = passed;
+            bool claim = first != 0;
+            if (first & stored) {                            // already stored
+                ss[idx] = (uint8_t)ST_EXISTS;
+                claim = false;
+            } else if (!first) {
+                b = Drain::bucket(v, b, d.group);
+                left = unread == d.group &&
+                       !(reach + d.group >= v.nb && b == first_bucket(v, (unsigned long long)key));
+                claim = !left && at != NONE;                 // only tombstones were free
+                if (!left && !claim) {                       // no free slot anywhere
+                    ss[idx] = (uint8_t)ST_OVERFLOW;
+                    cnts.over = 1;
+                }
+            }
+            if (claim) left = claim_slot(at, key, val, idx, b);
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int q = __popc(mask & lanes_below());
+            st.at[q] = b << 16 | (unsigned)idx;
+            st.free_at[q] = at;
+            st.key[q] = key;
+            if constexpr (T::MAP) st.val[q] = val;
+        }
+        top = __popc(mask);
+        reach += d.group;
+        __syncwarp();
+    }
+    __syncwarp();
+}
+
+// Erases the keys src.key(i), i < cnt, except those with src.skip(i) (later
+// occurrences: NOT_FOUND); statuses go to ss[i].  A failed swap means an equal
+// key of the same call erased the slot first: that key reports ERASED, this one
+// NOT_FOUND.
+template <int KIND, int BB, class Src>
+__device__ __forceinline__ void erase_run(const View &v, Src &src, int cnt, Stack<KIND, 2> &st, uint8_t *ss,
+                                          Counts &cnts) {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using Sl = Slots<KIND, BB>;
+    constexpr int LB = Sl::KRB;
+    const int lane = threadIdx.x & 31;
+    int next = 0, top = 0;
+    Key ahead = Key();
+    bool ahead_skip = false;
+    auto fetch = [&](int i) {
+        if (i >= cnt) return;
+        ahead = src.key(i);
+        ahead_skip = src.skip(i);
+    };
+    fetch(lane);
+    unsigned long long reach = 0;
+    const int few = v.nb >= 32 ? 16 : 0;     // a group's buckets are distinct
+    for (;; ++reach) {
+        Key key;
+        unsigned long long b = 0;
+        int idx;
+        bool act;
+        if (top < 32 && next < cnt) {
+            key = ahead;
+            idx = next + lane;
+            act = idx < cnt;
+            if (act && ahead_skip) {
+                ss[idx] = (uint8_t)ST_NOT_FOUND;
+                act = false;
+            }
+            next += 32;
+            fetch(next + lane);
+            const int side = side_index<KIND>(key);
+            if (act && side >= 0) {          // key equal to a marker: side slot
+                const bool won = atomicCAS(&v.hdr->side_present[side], 1u, 0u) == 1u;
+                cnts.del += won ? 1u : 0u;
+                ss[idx] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
+                act = false;
+            }
+            b = first_bucket(v, (unsigned long long)key);
+        } else if (top > few) {
+            const int take = top < 32 ? top : 32;
+            top -= take;
+            act = lane < take;
+            const int p = top + (act ? lane : 0);
+            const unsigned long long e = st.at[p];
+            key = st.key[p];
+            idx = (int)(e & 0xffffu);
+            b = e >> 16;
+        } else {
+            break;
+        }
+        __syncwarp();                        // entries are read before this step's survivors overwrite them
+        LaneWords<LB> lw;
+        if (act) lw.load(bucket_at<BB>(v, b));
+        bool left = false;
+        if (act) {
+            int hit = -1;
+            bool empty = false;
+#pragma unroll
+            for (int x = 0; x < Sl::SPB; ++x) {
+                const Key ks = slot_key<KIND, LB>(lw, x);
+                if (ks == key) hit = x;
+                empty |= ks == T::EMPTY;
+            }
+            if (hit >= 0) {
+                const bool won = cas_key<KIND>(Sl::key(v, b, hit), key, T::TOMB) == key;
+                if (won) note_claim_key<KIND>(v.hdr, key, -1);
+                ss[idx] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
+                cnts.del += won ? 1u : 0u;
+            } else {
+                b = next_bucket(v, b);
+                left = !empty && !came_round(v, (unsigned long long)key, b, reach);
+                if (!left) ss[idx] = (uint8_t)ST_NOT_FOUND;
+            }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int p = top + __popc(mask & lanes_below());
+            st.at[p] = b << 16 | (unsigned)idx;
+            st.key[p] = key;
+        }
+        top += __popc(mask);
+        __syncwarp();
+    }
+    while (top > 0) {
+        const Drain d(top);
+        const bool act = d.entry < top;
+        const int p = act ? d.entry : 0;
+        const unsigned long long e = st.at[p];
+        const Key key = st.key[p];
+        const int idx = (int)(e & 0xffffu);
+        unsigned long long b = e >> 16;
+        __syncwarp();
+        const int unread = d.unread(v, (unsigned long long)key, b, reach);
+        const unsigned long long mine = Drain::bucket(v, b, d.sub);
+        int hit = -1;
+        bool empty = false;
+        if (act && d.sub < unread) {
+            LaneWords<LB> lw;
+            lw.load(bucket_at<BB>(v, mine));
+#pragma unroll
+            for (int x = 0; x < Sl::SPB; ++x) {
+                const Key ks = slot_key<KIND, LB>(lw, x);
+                if (ks == key) hit = x;
+                empty |= ks == T::EMPTY;
+            }
+        }
+        const unsigned stop = d.ballot(hit >= 0 || empty);
+        bool left = false;
+        if (act && stop) {
+            if (d.sub == __ffs(stop) - 1) {
+                const bool won = hit >= 0 && cas_key<KIND>(Sl::key(v, mine, hit), key, T::TOMB) == key;
+                if (won) note_claim_key<KIND>(v.hdr, key, -1);
+                ss[idx] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
+                cnts.del += won ? 1u : 0u;
+            }
+        } else if (act && d.sub == 0) {
+            left = unread == d.group;
+            b = Drain::bucket(v, b, d.group);
+            left = left && !(reach + d.group >= v.nb && b == first_bucket(v, (unsigned long long)key));
+            if (!left) ss[idx] = (uint8_t)ST_NOT_FOUND;
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int q = __popc(mask & lanes_below());
+            st.at[q] = b << 16 | (unsigned)idx;
+            st.key[q] = key;
+        }
+        top = __popc(mask);
+        reach += d.group;
+        __syncwarp();
+    }
+    __syncwarp();
+}
+
+// A run of the caller's arrays, in order.
+template <int KIND>
+struct ArraySrc {
+    using Key = typename Traits<KIND>::Key;
+    using Val = typename Traits<KIND>::Val;
+    const Key *keys;
+    const Val *vals;
+    const uint8_t *skips;
+    __device__ __forceinline__ Key key(int i) const { return ld_stream(keys + i); }
+    __device__ __forceinline__ Val val(int i) const { return ld_stream(vals + i); }
+    __device__ __forceinline__ bool skip(int i) const { return skips && ld_stream(skips + i); }
+};
+
+// Shared memory of one warp for runs of R keys.
+template <int KIND, int OP, int R>
+struct alignas(16) WarpRun {
+    Stack<KIND, OP> stack;
+    typename Traits<KIND>::Val vals[Traits<KIND>::MAP && OP == 1 ? R : 1];
+    uint8_t st[R];
+};
+
+// The counts of a block's warps, added up in shared memory and moved to the
+// header by the warp that finishes last.  Atomics on the one header line go one
+// after another (1.5-3 ns each): with one per warp, 2^26 erases in runs of 64
+// keys ran at 15.3 G/s instead of 21.4, and 10^6 L2-resident set erases at 21.6
+// instead of 32.4.
+struct BlockCounts {
+    unsigned ins, new_slot, del, over, done;
+    // by every thread of the block, before any flush
+    __device__ __forceinline__ void init() {
+        if (threadIdx.x == 0) ins = new_slot = del = over = done = 0u;
+        __syncthreads();
+    }
+    // by all lanes of a warp; `warps` warps of the block do it
+    __device__ __forceinline__ void flush(const View &v, const Counts &c, int warps) {
+        __syncwarp();
+        const uint32_t w_ins = __reduce_add_sync(0xffffffffu, c.ins);
+        const uint32_t w_new = __reduce_add_sync(0xffffffffu, c.new_slot);
+        const uint32_t w_del = __reduce_add_sync(0xffffffffu, c.del);
+        const uint32_t w_over = __reduce_or_sync(0xffffffffu, c.over);
+        if ((threadIdx.x & 31) == 0) {
+            if (w_ins) atomicAdd(&ins, w_ins);
+            if (w_new) atomicAdd(&new_slot, w_new);
+            if (w_del) atomicAdd(&del, w_del);
+            if (w_over) atomicOr(&over, 1u);
+            __threadfence_block();
+            if (atomicAdd(&done, 1u) == (unsigned)warps - 1u) {
+                __threadfence_block();
+                const long long d = (long long)atomicAdd(&ins, 0u) - (long long)atomicAdd(&del, 0u);
+                const unsigned used = atomicAdd(&new_slot, 0u);
+                if (d) atomicAdd(&v.hdr->live, (unsigned long long)d);
+                if (used) atomicAdd(&v.hdr->used, (unsigned long long)used);
+                if (atomicAdd(&over, 0u)) atomicOr(&v.hdr->err, ERR_OVERFLOW);
+            }
+        }
+    }
+};
+
+// The range kernels: warp w of the grid takes keys [w * run, w * run + run),
+// run <= R.  5 blocks of 256 threads (51 registers) keep every kind's state
+// without spills; at 6 (40 registers, 20-40 bytes spilled) lookups and inserts
+// beyond L2 are 2-6 % slower, at 8 (32) 10-20 %.
+template <int KIND, int BB, int OP, int R>
+__global__ void __launch_bounds__(256, 5)
+k_run(View v, const typename Traits<KIND>::Key *keys, const typename Traits<KIND>::Val *vals, const uint8_t *skip,
+      long long n, int run, uint8_t *out, typename Traits<KIND>::Val *vals_out) {
+    using T = Traits<KIND>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ BlockCounts sum;
+    WarpRun<KIND, OP, R> &w = reinterpret_cast<WarpRun<KIND, OP, R> *>(smem)[threadIdx.x >> 5];
+    if constexpr (OP != 1) sum.init();
+    const long long w0 = (long long)blockIdx.x * (blockDim.x >> 5);
+    const long long c0 = (w0 + (threadIdx.x >> 5)) * run;
+    if (c0 >= n) return;
+    const int cnt = (int)(n - c0 < run ? n - c0 : run);
+    debug_range(v, c0, cnt, n);
+    ArraySrc<KIND> src{keys + c0, vals + c0, skip ? skip + c0 : nullptr};
+    Counts cnts;
+    if constexpr (OP == 0) insert_run<KIND, BB>(v, src, cnt, w.stack, w.st, cnts);
+    else if constexpr (OP == 1) find_run<KIND, BB>(v, src, cnt, w.stack, w.st, w.vals);
+    else erase_run<KIND, BB>(v, src, cnt, w.stack, w.st, cnts);
+    for (int i = threadIdx.x & 31; i < cnt; i += 32) {
+        if (out) st_stream(out + c0 + i, w.st[i]);
+        if constexpr (OP == 1 && T::MAP) {
+            if (vals_out) st_stream(vals_out + c0 + i, w.vals[i]);
+        }
+    }
+    if constexpr (OP != 1) {
+        const long long busy = (n + run - 1) / run - w0;     // warps of this block with keys
+        sum.flush(v, cnts, (int)(busy < (blockDim.x >> 5) ? busy : (blockDim.x >> 5)));
+    }
 }
 
 // Streaming map lookup by lane pairs: the two lanes of a pair handle one key.
@@ -245,7 +815,7 @@ k_find_stream(View v, const typename Traits<KIND>::Key *keys, long long n, uint8
 // its value separately.  The pair keeps identical state and control flow and
 // exchanges the comparison masks with shuffles.
 template <int KIND, int BB, int KPT, int S>
-__global__ void __launch_bounds__(256, HC_STREAM_FIND_MINB)
+__global__ void __launch_bounds__(256)
 k_find_pair(View v, const typename Traits<KIND>::Key *keys, long long n, uint8_t *found,
             typename Traits<KIND>::Val *vals_out) {
     using T = Traits<KIND>;
@@ -383,314 +953,6 @@ k_find_pair(View v, const typename Traits<KIND>::Key *keys, long long n, uint8_t
         if (found) st_stream(found + c0 + i, sf[i]);
         if (vals_out) st_stream(vals_out + c0 + i, sv[i]);
     }
-}
-
-// Streaming insert: the same staging and refilling as k_find_stream.  Within
-// one round every slot first decides whether it claims, then all claiming
-// slots issue their compare-and-swap together, so the atomics of different
-// keys overlap.  Statuses collect in shared memory and leave in coalesced
-// stores; counters leave with one atomic per warp.  Equal keys inside a warp
-// are not folded here (folding is a lock-step option).
-template <int KIND, int BB, int KPT, int S>
-__device__ __forceinline__ void insert_stream_chunk(const View &v, const typename Traits<KIND>::Key *keys,
-                                                    const typename Traits<KIND>::Val *vals, long long c0, int m,
-                                                    uint8_t *status, const uint8_t *skip) {
-    using T = Traits<KIND>;
-    using Key = typename T::Key;
-    using Val = typename T::Val;
-    using Sl = Slots<KIND, BB>;
-    using Lay = Layout<KIND, BB, Sl::KRB>;
-    constexpr int LB = Sl::KRB;
-    constexpr int SPL = Sl::SPB;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int nt = blockDim.x;
-    const int chunk = nt * KPT;
-    Key *sk = reinterpret_cast<Key *>(smem);
-    Val *sv = reinterpret_cast<Val *>(smem + (size_t)chunk * sizeof(Key));
-    uint8_t *ss = smem + (size_t)chunk * (sizeof(Key) + sizeof(Val));
-
-    Stage<Key, KPT> gk;
-    Stage<Val, KPT> gv;
-    Stage<uint8_t, KPT> gs;
-    gk.load(keys + c0, m);
-    if constexpr (T::MAP) gv.load(vals + c0, m);
-    if (skip) gs.load(skip + c0, m);
-    __syncthreads();                         // the staging of a previous chunk is no longer read
-    gk.store(sk, m);
-    if constexpr (T::MAP) gv.store(sv, m);
-    // result bytes: ST_EXISTS for keys a find reported present, 0xFF (to do)
-    if (skip) gs.store(ss, m, [](uint8_t f) { return f ? (uint8_t)ST_EXISTS : (uint8_t)0xFF; });
-    else
-        for (int i = threadIdx.x; i < m; i += nt) ss[i] = 0xFF;
-    __syncthreads();
-
-    Counts cnt;
-    int idx[S];
-    Key key[S];
-    unsigned long long b[S], ffb[S];
-    uint32_t probes[S], restarts[S], ffs_slot[S];
-    bool ff_empty[S];
-    int next = 0;
-    uint32_t active = 0;
-    auto take = [&](int s) {
-        while (next < KPT) {
-            const int i = threadIdx.x + (next++) * nt;
-            if (i >= m) { next = KPT; break; }
-            if (ss[i] != 0xFF) continue;                       // reported present by a find
-            const Key k = sk[i];
-            const int side = side_index<KIND>(k);
-            if (side >= 0) {                                   // key equal to a marker: side slot
-                const bool won = atomicCAS(&v.hdr->side_present[side], 0u, 1u) == 0u;
-                if (won) {
-                    if constexpr (T::MAP) v.hdr->side_val[side] = (unsigned long long)sv[i];
-                    ++cnt.ins;
-                }
-                ss[i] = won ? (uint8_t)ST_INSERTED : (uint8_t)ST_EXISTS;
-                continue;
-            }
-            idx[s] = i;
-            key[s] = k;
-            b[s] = first_bucket(v, (unsigned long long)k);
-            probes[s] = 0;
-            restarts[s] = 0;
-            ffb[s] = ~0ull;
-            active |= 1u << s;
-            return;
-        }
-    };
-#pragma unroll
-    for (int s = 0; s < S; ++s) take(s);
-    while (active) {
-        LaneWords<LB> lw[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-            if (active >> s & 1u) lw[s].load(bucket_at<BB>(v, b[s]));
-        uint32_t claiming = 0;
-        uint32_t finished = 0;
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(active >> s & 1u)) continue;
-            uint32_t lm = 0, le = 0, lt = 0;
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                const Key ks = slot_key<KIND, LB>(lw[s], q);
-                lm |= (uint32_t)(ks == key[s]) << q;
-                le |= (uint32_t)(ks == T::EMPTY) << q;
-                lt |= (uint32_t)(ks == T::TOMB) << q;
-            }
-            if (lm) {                                           // already stored
-                ss[idx[s]] = ST_EXISTS;
-                finished |= 1u << s;
-                continue;
-            }
-            if (ffb[s] == ~0ull) {                              // first free slot, rotated scan
-                lt &= claimable<KIND, BB, LB>(v, b[s], 0);
-                const uint32_t lf = le | lt;
-                if (lf) {
-                    const int rot = v.rotate ? slot_rotation<Lay::SPB>(key[s]) : 0;
-                    const uint32_t hi = lf & (Lay::ALL & ~((1u << rot) - 1u));
-                    const int q = __ffs(hi ? hi : lf) - 1;
-                    ffb[s] = b[s];
-                    ffs_slot[s] = q;
-                    ff_empty[s] = (le >> q) & 1u;
-                }
-            }
-            if (le) {
-                claiming |= 1u << s;
-            } else if (++probes[s] >= v.nb) {
-                if (ffb[s] == ~0ull) {                          // no free slot anywhere
-                    ss[idx[s]] = ST_OVERFLOW;
-                    cnt.over = 1;
-                    finished |= 1u << s;
-                } else {
-                    claiming |= 1u << s;                        // only tombstones were free
-                }
-            } else {
-                b[s] = next_bucket(v, b[s]);
-            }
-        }
-        Key old[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-            if (claiming >> s & 1u)
-                old[s] = cas_key<KIND>(Slots<KIND, BB>::key(v, ffb[s], ffs_slot[s]), ff_empty[s] ? T::EMPTY : T::TOMB,
-                                       key[s]);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(claiming >> s & 1u)) continue;
-            const Key expect = ff_empty[s] ? T::EMPTY : T::TOMB;
-            if (old[s] == expect) {
-                if constexpr (T::MAP) {
-                    store_val<KIND, BB>(v, ffb[s], ffs_slot[s], (unsigned long long)sv[idx[s]]);
-                    note_claim_key<KIND>(v.hdr, key[s], (long long)(ffb[s] * SPL) + ffs_slot[s]);
-                }
-                ss[idx[s]] = ST_INSERTED;
-                ++cnt.ins;
-                cnt.new_slot += ff_empty[s] ? 1u : 0u;
-                finished |= 1u << s;
-            } else if (old[s] == key[s]) {
-                ss[idx[s]] = ST_EXISTS;                         // an equal key won the race
-                finished |= 1u << s;
-            } else if (++restarts[s] > kMaxRestarts) {
-                atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
-                ss[idx[s]] = ST_OVERFLOW;
-                cnt.over = 1;
-                finished |= 1u << s;
-            } else {                                            // lost the slot to another key
-                b[s] = first_bucket(v, (unsigned long long)key[s]);
-                probes[s] = 0;
-                ffb[s] = ~0ull;
-            }
-        }
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (finished >> s & 1u) {
-                active &= ~(1u << s);
-                take(s);
-            }
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += nt)
-        if (status) st_stream(status + c0 + i, ss[i]);
-    flush_counts(v, cnt);
-}
-
-template <int KIND, int BB, int KPT, int S>
-__global__ void __launch_bounds__(256, HC_STREAM_INSERT_MINB)
-k_insert_stream(View v, const typename Traits<KIND>::Key *keys, const typename Traits<KIND>::Val *vals, long long n,
-                uint8_t *status, const uint8_t *skip) {
-    const long long chunk = (long long)blockDim.x * KPT;
-    const long long c0 = (long long)blockIdx.x * chunk;
-    const int m = (int)(n - c0 < chunk ? n - c0 : chunk);
-    debug_range(v, c0, m, n);
-    insert_stream_chunk<KIND, BB, KPT, S>(v, keys, vals, c0, m, status, skip);
-}
-
-// Streaming erase: the staging and refilling of k_find_stream; a slot that
-// finds its key joins the round's compare-and-swap (key -> TOMB) with the
-// other slots that found theirs.  A failed swap means an equal key of the
-// same call erased the slot first: that key reports ERASED, this one
-// NOT_FOUND, as in the lock-step form.  Keys flagged in `skip` report
-// NOT_FOUND without a probe (the later occurrences of a key in the ordered
-// erase).
-template <int KIND, int BB, int KPT, int S>
-__device__ __forceinline__ void erase_stream_chunk(const View &v, const typename Traits<KIND>::Key *keys, long long c0, int m,
-                                                   uint8_t *status, const uint8_t *skip) {
-    using T = Traits<KIND>;
-    using Key = typename T::Key;
-    using Sl = Slots<KIND, BB>;
-    constexpr int LB = Sl::KRB;
-    constexpr int SPL = Sl::SPB;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int nt = blockDim.x;
-    const int chunk = nt * KPT;
-    Key *sk = reinterpret_cast<Key *>(smem);
-    uint8_t *ss = smem + (size_t)chunk * sizeof(Key);
-
-    Stage<Key, KPT> gk;
-    Stage<uint8_t, KPT> gs;
-    gk.load(keys + c0, m);
-    if (skip) gs.load(skip + c0, m);
-    __syncthreads();                         // the staging of a previous chunk is no longer read
-    gk.store(sk, m);
-    // result bytes: NOT_FOUND for the later occurrences of a key, 0xFF (to do)
-    if (skip) gs.store(ss, m, [](uint8_t f) { return f ? (uint8_t)ST_NOT_FOUND : (uint8_t)0xFF; });
-    else
-        for (int i = threadIdx.x; i < m; i += nt) ss[i] = 0xFF;
-    __syncthreads();
-
-    Counts cnt;
-    int idx[S];
-    Key key[S];
-    unsigned long long b[S];
-    uint32_t probes[S], hit_slot[S];
-    int next = 0;
-    uint32_t active = 0;
-    auto take = [&](int s) {
-        while (next < KPT) {
-            const int i = threadIdx.x + (next++) * nt;
-            if (i >= m) { next = KPT; break; }
-            if (ss[i] != 0xFF) continue;                       // a later occurrence: NOT_FOUND
-            const Key k = sk[i];
-            const int side = side_index<KIND>(k);
-            if (side >= 0) {                                   // key equal to a marker: side slot
-                const bool won = atomicCAS(&v.hdr->side_present[side], 1u, 0u) == 1u;
-                cnt.del += won ? 1u : 0u;
-                ss[i] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
-                continue;
-            }
-            idx[s] = i;
-            key[s] = k;
-            b[s] = first_bucket(v, (unsigned long long)k);
-            probes[s] = 0;
-            active |= 1u << s;
-            return;
-        }
-    };
-#pragma unroll
-    for (int s = 0; s < S; ++s) take(s);
-    while (active) {
-        LaneWords<LB> lw[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-            if (active >> s & 1u) lw[s].load(bucket_at<BB>(v, b[s]));
-        uint32_t hitting = 0, finished = 0;
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(active >> s & 1u)) continue;
-            uint32_t lm = 0, le = 0;
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                const Key ks = slot_key<KIND, LB>(lw[s], q);
-                lm |= (uint32_t)(ks == key[s]) << q;
-                le |= (uint32_t)(ks == T::EMPTY) << q;
-            }
-            if (lm) {
-                hit_slot[s] = __ffs(lm) - 1;
-                hitting |= 1u << s;
-            } else if (le || ++probes[s] >= v.nb) {
-                ss[idx[s]] = ST_NOT_FOUND;
-                finished |= 1u << s;
-            } else {
-                b[s] = next_bucket(v, b[s]);
-            }
-        }
-        Key old[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-            if (hitting >> s & 1u) old[s] = cas_key<KIND>(Sl::key(v, b[s], hit_slot[s]), key[s], T::TOMB);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(hitting >> s & 1u)) continue;
-            const bool won = old[s] == key[s];
-            if (won) note_claim_key<KIND>(v.hdr, key[s], -1);
-            ss[idx[s]] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
-            cnt.del += won ? 1u : 0u;
-            finished |= 1u << s;
-        }
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (finished >> s & 1u) {
-                active &= ~(1u << s);
-                take(s);
-            }
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += nt)
-        if (status) st_stream(status + c0 + i, ss[i]);
-    flush_counts(v, cnt);
-}
-
-template <int KIND, int BB, int KPT, int S>
-__global__ void __launch_bounds__(256, HC_STREAM_ERASE_MINB)
-k_erase_stream(View v, const typename Traits<KIND>::Key *keys, long long n, uint8_t *status, const uint8_t *skip) {
-    const long long chunk = (long long)blockDim.x * KPT;
-    const long long c0 = (long long)blockIdx.x * chunk;
-    const int m = (int)(n - c0 < chunk ? n - c0 : chunk);
-    debug_range(v, c0, m, n);
-    erase_stream_chunk<KIND, BB, KPT, S>(v, keys, c0, m, status, skip);
 }
 
 }  // namespace hc

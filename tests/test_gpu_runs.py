@@ -1,0 +1,84 @@
+"""The warp-run kernels where their probe loops end: tables without an EMPTY
+slot, probes that come round the whole table, and batches at the edges of a
+step (32 keys) and of a run."""
+import numpy as np
+import pytest
+
+from gpu_pair import Pair, random_keys, value_for
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+KINDS = (O.SET_U32, O.SET_U64, O.MAP_I64_I32, O.MAP_U64_U64)
+SPB = {O.SET_U32: lambda bb: bb // 4, O.SET_U64: lambda bb: bb // 8, O.MAP_I64_I32: lambda bb: bb // 16,
+       O.MAP_U64_U64: lambda bb: bb // 16}
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("bb", (32, 64, 128))
+@pytest.mark.parametrize("nb", (1, 2, 31, 32, 33, 65))
+@pytest.mark.parametrize("pad", (0, 1))
+def test_full_table_and_tombstones_only(kind, bb, nb, pad):
+    """32 buckets and more share the end of a run among several lanes per key;
+    fewer do not.  A full table answers absent keys after reading every bucket
+    once, refuses inserts, and takes them again once its slots are tombstones;
+    `pad` leaves the last bucket's last slot outside the capacity."""
+    slots = nb * SPB[kind](bb) - pad
+    if slots < 1:
+        pytest.skip("no slot")
+    rng = np.random.default_rng(1000 * nb + 10 * bb + kind)
+    keys = np.unique(random_keys(kind, 3 * slots + 40, rng))
+    rng.shuffle(keys)
+    stored, other = keys[:slots], keys[slots:2 * slots + 20]
+    p = Pair(kind, slots, bucket_bytes=bb)
+    try:
+        p.insert(stored, value_for(kind, stored))
+        p.find(np.concatenate([stored, other]))
+        p.insert(other[:7], value_for(kind, other[:7]))                 # every one overflows
+        p.insert(np.concatenate([stored, other]), value_for(kind, np.concatenate([stored, other]), salt=1))
+        p.check()
+        p.erase(np.concatenate([other, stored]))
+        p.find(np.concatenate([stored, other]))                         # tombstones only
+        p.erase(other)
+        p.insert(other[:slots], value_for(kind, other[:slots]))         # reuses them
+        p.check()
+        p.erase(other[:slots:2])
+        p.insert(np.concatenate([other[:slots]] * 2), value_for(kind, np.concatenate([other[:slots]] * 2), salt=2))
+        p.check()
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("bb", (32, 128))
+@pytest.mark.parametrize("kpt", (4, 8))
+def test_batches_at_the_edges_of_steps_and_runs(kind, bb, kpt):
+    """Batch sizes around a step and a run, with arrays that start one element
+    off a 16-byte boundary, at a load factor with long probe sequences."""
+    import torch
+
+    from paper_1908_05936_gb300.table import to_device, to_numpy
+    rng = np.random.default_rng(bb + kpt + kind)
+    p = Pair(kind, 9000, bucket_bytes=bb)
+    for op in (0, 1, 2):
+        p.g.set_launch(op, keys_per_group=kpt, block=128)
+    keys = np.unique(random_keys(kind, 12000, rng))
+    rng.shuffle(keys)
+    try:
+        at = 0
+        for n in (1, 31, 32, 33, 32 * kpt - 1, 32 * kpt, 32 * kpt + 1, 4 * 32 * kpt + 1, 6000):
+            k = keys[at:at + n]
+            at += n
+            p.insert(k, value_for(kind, k))
+            p.find(np.concatenate([k, keys[-n:]]))
+            dev = torch.empty(n + 1, dtype=to_device(k).dtype, device="cuda")[1:]
+            dev.copy_(to_device(k))
+            f, v = p.g.find(dev)
+            of, ov = p.o.find(k)
+            assert np.array_equal(to_numpy(f, np.uint8), of)
+            if p.is_map:
+                assert np.array_equal(to_numpy(v, O.VAL_DTYPE[kind]), ov)
+            p.erase(k[::4])
+        p.check()
+    finally:
+        p.close()

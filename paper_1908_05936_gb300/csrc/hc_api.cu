@@ -67,19 +67,6 @@ int sm_count_of(int dev) {
     return cache[dev];
 }
 
-long long l2_bytes_of(int dev) {
-    static std::mutex mu;
-    static long long cache[64] = {0};
-    std::lock_guard<std::mutex> g(mu);
-    if (dev < 0 || dev >= 64) return 128ll << 20;
-    if (!cache[dev]) {
-        int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrL2CacheSize, dev) != cudaSuccess || n <= 0) n = 128 << 20;
-        cache[dev] = n;
-    }
-    return cache[dev];
-}
-
 hc_rc check_config(int kind, const hc_config *cfg, int *bb, int *hash_mode, unsigned long long *seed) {
     *bb = 32;
     *hash_mode = HC_HASH_MIX64;
@@ -135,6 +122,142 @@ cudaError_t dispatch_range(int kind, int op, const hc::View &v, int bb, const vo
         case HC_MAP_I64_I32: return hc::map_i64_i32_range(op, v, bb, keys, vals, n, out, vals_out, sh, skip, s);
         default: return hc::map_u64_u64_range(op, v, bb, keys, vals, n, out, vals_out, sh, skip, s);
     }
+}
+
+cudaError_t dispatch_bulk(int kind, int op, const hc::View &v, int bb, const void *keys, const void *vals, long long n,
+                          uint8_t *out, void *vals_out, int parts, void *scratch, cudaStream_t s) {
+    switch (kind) {
+        case HC_SET_U32: return hc::set_u32_bulk(op, v, bb, keys, vals, n, out, vals_out, parts, scratch, s);
+        case HC_SET_U64: return hc::set_u64_bulk(op, v, bb, keys, vals, n, out, vals_out, parts, scratch, s);
+        case HC_MAP_I64_I32: return hc::map_i64_i32_bulk(op, v, bb, keys, vals, n, out, vals_out, parts, scratch, s);
+        default: return hc::map_u64_u64_bulk(op, v, bb, keys, vals, n, out, vals_out, parts, scratch, s);
+    }
+}
+
+// Scratch of the bulk calls: a memory pool per device, so that a call takes
+// and gives back its scratch in stream order (several threads, streams and
+// tables each hold their own).  The pool keeps at most kPoolKeep bytes between
+// calls and nothing once the device's last table is gone.
+constexpr unsigned long long kPoolKeep = 1536ull << 20;   // a 2^26-key insert's scratch is 1280 MB
+
+struct ScratchPool {
+    std::mutex mu;
+    cudaMemPool_t pool = nullptr;
+    long long tables = 0;
+};
+
+ScratchPool &scratch_pool(int dev) {
+    static ScratchPool pools[64];
+    return pools[dev];
+}
+
+cudaMemPool_t pool_of(int dev) {
+    if (dev < 0 || dev >= 64) return nullptr;
+    ScratchPool &p = scratch_pool(dev);
+    std::lock_guard<std::mutex> g(p.mu);
+    if (!p.pool) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        unsigned long long keep = kPoolKeep;
+        int no = 0;
+        if (cudaMemPoolCreate(&p.pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+            // independent streams stay independent: no reuse that would make one wait for another
+            cudaMemPoolSetAttribute(p.pool, cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess) {
+            (void)cudaGetLastError();
+            if (p.pool) cudaMemPoolDestroy(p.pool);
+            p.pool = nullptr;
+        }
+    }
+    return p.pool;
+}
+
+// A table more (+1) or less (-1) on the device; the last one gives the pool's
+// memory back (its work is done: cudaFree has waited for the device).
+void count_table(int dev, int d) {
+    if (dev < 0 || dev >= 64) return;
+    ScratchPool &p = scratch_pool(dev);
+    std::lock_guard<std::mutex> g(p.mu);
+    p.tables += d;
+    if (p.tables == 0 && p.pool) (void)cudaMemPoolTrimTo(p.pool, 0);
+}
+
+// cudaMalloc of a table; when memory is short, again without the pool's.
+cudaError_t table_malloc(void **mem, long long bytes, int dev) {
+    cudaError_t e = cudaMalloc(mem, bytes);
+    if (e == cudaErrorMemoryAllocation && dev >= 0 && dev < 64) {
+        ScratchPool &p = scratch_pool(dev);
+        std::lock_guard<std::mutex> g(p.mu);
+        if (p.pool) {
+            (void)cudaGetLastError();
+            (void)cudaDeviceSynchronize();
+            (void)cudaMemPoolTrimTo(p.pool, 0);
+            e = cudaMalloc(mem, bytes);
+        }
+    }
+    return e;
+}
+
+// Whether a call of n keys runs as a bulk call (hc_bulk.cuh).  Splitting and
+// joining cost about 0.009 ns a key; what they buy is a table read part by
+// part, so the line is drawn in keys per 128-byte line of the table (x), and
+// only for tables beyond the reach of the address translation.  Measured
+// against the warp runs (2^24-2^30 slots, load factors 0.4-0.8, 32- to 128-byte
+// buckets, bulk time / run time inverted):
+//   maps   lookups  x = 0.5: present 1.07-1.3, absent 0.73-1.0; 1: 1.25-1.5 and
+//                   0.87-1.4; 2: 1.5-1.7 and 1.1-1.2
+//   sets   lookups  x = 1: 0.9-1.04 and 0.98-2.0; 4: 1.2 and 1.28
+//   inserts         x = 0.25: 0.9-1.3; 0.5: 0.97-1.35; 1: 1.16-1.8; 2: 1.5-1.8
+//   erases          x = 0.5: 0.93-1.2; 1: 1.15-1.6
+//   512 MB tables   about twice the x for the same gain; 256 MB: never.
+bool bulk_pays(const hc_table *t, int op, long long n) {
+    const long long bytes = (long long)t->view.nb * t->bucket_bytes;
+    if (n < (1ll << 21) || bytes < (512ll << 20)) return false;
+    const double x = (double)n * 128.0 / (double)bytes;
+    const double large = op == hc::OP_INSERT ? 0.5 : op == hc::OP_ERASE ? 1.0 : is_map(t->kind) ? 1.25 : 1.5;
+    return x >= (bytes < (768ll << 20) ? 2.0 * large + 1.0 : large);
+}
+
+// Device memory (not mapped host memory, which the splitting pass would read twice).
+bool on_device(const void *p) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
+}
+
+// Runs the call as a bulk call if that pays and its scratch can be had: a
+// stream that is capturing, or a device without the memory, keeps the range
+// kernels.  *done says whether it ran.
+cudaError_t try_bulk(hc_table *t, int op, const hc::View &v, const void *keys, const void *vals, long long n,
+                     uint8_t *out, void *vals_out, cudaStream_t s, bool *done) {
+    *done = false;
+    if (t->shape_set[op] || !bulk_pays(t, op, n) || !on_device(keys) || (vals && !on_device(vals))) return cudaSuccess;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();
+        return cudaSuccess;
+    }
+    cudaMemPool_t pool = pool_of(t->device);
+    if (!pool) return cudaSuccess;
+    // parts of about 32 MB: two of them and the keys in flight stay in L2
+    const long long bytes = (long long)v.nb * t->bucket_bytes;
+    const int parts = (int)std::min<long long>(hc::kBulkParts, (bytes + (32ll << 20) - 1) / (32ll << 20));
+    void *scratch = nullptr;
+    const long long need = hc::bulk_scratch(nullptr, nullptr, std::min(n, hc::kBulkPiece), parts, key_bytes(t->kind),
+                                            val_bytes(t->kind), op);
+    if (cudaMallocFromPoolAsync(&scratch, need, pool, s) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return cudaSuccess;
+    }
+    *done = true;
+    const cudaError_t e = dispatch_bulk(t->kind, op, v, t->bucket_bytes, keys, vals, n, out, vals_out, parts, scratch, s);
+    const cudaError_t f = cudaFreeAsync(scratch, s);
+    return e != cudaSuccess ? e : f;
 }
 
 cudaError_t dispatch_clear(const hc_table *t, const hc::View &v, long long phys, long long cap, cudaStream_t s) {
@@ -202,8 +325,12 @@ hc_rc run_range(hc_table *t, int op, const void *keys, const void *vals, long lo
     sh.sms = sm_count_of(t->device);
     hc::View v = t->view;
     v.rotate = n > (long long)v.nb ? 1 : 0;        // several inserters per bucket: spread them
-    cudaError_t e = dispatch_range(t->kind, op, v, t->bucket_bytes, keys, is_map(t->kind) ? vals : nullptr, n,
-                                   out, is_map(t->kind) ? vals_out : nullptr, sh, skip, s);
+    const void *in = is_map(t->kind) && op == hc::OP_INSERT ? vals : nullptr;
+    void *vo = is_map(t->kind) ? vals_out : nullptr;
+    bool done = false;
+    cudaError_t e = cudaSuccess;
+    if (!skip) e = try_bulk(t, op, v, keys, in, n, out, vo, s, &done);
+    if (!done) e = dispatch_range(t->kind, op, v, t->bucket_bytes, keys, in, n, out, vo, sh, skip, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the range kernel");
     return HC_OK;
 }
@@ -338,7 +465,7 @@ hc_rc hc_create(hc_table **out, int32_t kind, int64_t slots, const hc_config *cf
     t->bytes = g.bytes;
     t->bucket_bytes = bb;
     HC_CUDA(cudaGetDevice(&t->device), "cudaGetDevice");
-    cudaError_t e = cudaMalloc(&t->d_mem, g.bytes);
+    cudaError_t e = table_malloc(&t->d_mem, g.bytes, t->device);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         delete t;
@@ -353,6 +480,7 @@ hc_rc hc_create(hc_table **out, int32_t kind, int64_t slots, const hc_config *cf
         delete t;
         return cuda_fail(e, "initialising the table");
     }
+    count_table(t->device, 1);
     *out = t;
     return HC_OK;
 }
@@ -371,6 +499,7 @@ hc_rc hc_destroy(hc_table *t) {
         }
         cudaStreamDestroy(t->copy_stream);
     }
+    count_table(t->device, -1);
     delete t;
     if (e != cudaSuccess) return cuda_fail(e, "cudaFree");
     return HC_OK;
@@ -508,7 +637,7 @@ hc_rc hc_rehash(hc_table *t, int64_t new_slots, void *stream) {
         return fail(HC_ERR_ARG, "new_slots %lld is below the %lld stored keys", (long long)new_slots, regular);
     const Geometry g = geometry(t->kind, new_slots, t->bucket_bytes);
     void *mem = nullptr;
-    cudaError_t e = cudaMalloc(&mem, g.bytes);
+    cudaError_t e = table_malloc(&mem, g.bytes, t->device);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return fail(HC_ERR_OOM, "cudaMalloc of %lld bytes failed: %s", (long long)g.bytes, cudaGetErrorString(e));

@@ -27,6 +27,8 @@ struct LaunchShape {
     cudaError_t NAME##_range(int op, const View &v, int bb, const void *keys, const void *vals, long long n,        \
                              uint8_t *out, void *vals_out, const LaunchShape &sh, const uint8_t *skip,              \
                              cudaStream_t s);                                                                       \
+    cudaError_t NAME##_bulk(int op, const View &v, int bb, const void *keys, const void *vals, long long n,         \
+                            uint8_t *out, void *vals_out, int parts, void *scratch, cudaStream_t s);                \
     cudaError_t NAME##_clear(const View &v, unsigned long long phys, unsigned long long cap, int bb, int sms,       \
                              cudaStream_t s);                                                                       \
     cudaError_t NAME##_rehash(const View &ov, unsigned long long ophys, const View &nv, int bb, int sms,            \
@@ -38,6 +40,42 @@ HC_DECLARE_KIND(map_i64_i32)
 HC_DECLARE_KIND(map_u64_u64)
 
 #undef HC_DECLARE_KIND
+
+// Bulk calls (hc_bulk.cuh): keys per chunk and per piece, parts at most.
+constexpr int kBulkChunk = 4096;
+constexpr long long kBulkPiece = 1ll << 26;
+constexpr int kBulkParts = 512;
+
+// Scratch of a piece of n keys, in the order of the members; every array
+// starts on a 256-byte boundary.
+// (A value is never wider than its key.)
+struct BulkScratch {
+    void *keys;              // keys in chunk order; a lookup puts a key's value over it
+    void *vals;              // an insert's values in chunk order
+    uint16_t *order;         // chunk position each one came from
+    uint8_t *out;            // results in chunk order
+    uint16_t *offs;          // chunks x (parts + 1): where each part begins in its chunk
+};
+
+inline long long bulk_align(long long b) { return (b + 255) / 256 * 256; }
+
+inline long long bulk_scratch(BulkScratch *out, unsigned char *base, long long n, int parts, int kb, int vb, int op) {
+    const long long chunks = (n + kBulkChunk - 1) / kBulkChunk;
+    long long at = 0;
+    auto take = [&](long long bytes) {
+        unsigned char *p = base + at;
+        at += bulk_align(bytes);
+        return p;
+    };
+    BulkScratch s;
+    s.keys = take(n * kb);
+    s.vals = take(op == OP_INSERT ? n * vb : 0);
+    s.order = reinterpret_cast<uint16_t *>(take(n * 2));
+    s.out = take(n);
+    s.offs = reinterpret_cast<uint16_t *>(take(chunks * (parts + 1) * 2));
+    if (out) *out = s;
+    return at;
+}
 
 // hc_predicate as the selection kernel takes it.
 struct SelectPred {

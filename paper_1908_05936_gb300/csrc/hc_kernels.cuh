@@ -3,6 +3,7 @@
 // kind by hc_kind_*.cu.
 #pragma once
 
+#include "hc_bulk.cuh"
 #include "hc_core.cuh"
 #include "hc_internal.h"
 #include "hc_stream.cuh"
@@ -282,6 +283,72 @@ cudaError_t launch_range(int op, const View &v, int bucket_bytes, const void *ke
     }
 }
 
+// The three passes of a bulk call on one piece of n <= kBulkPiece keys.  64
+// threads (two warps) per probing block: 24 blocks per SM hold 40 registers.
+template <int KIND, int BB, int OP>
+cudaError_t launch_bulk_op(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
+                           int parts, void *scratch, cudaStream_t s) {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using Val = typename T::Val;
+    constexpr bool VIN = T::MAP && OP == OP_INSERT;
+    constexpr int NT = 64, R = 256, MINB = 24;
+    BulkScratch sc;
+    bulk_scratch(&sc, static_cast<unsigned char *>(scratch), n, parts, (int)sizeof(Key), T::MAP ? (int)sizeof(Val) : 0, OP);
+    const int chunks = (int)((n + kBulkChunk - 1) / kBulkChunk);
+    const unsigned long long part_mul = (unsigned long long)(((unsigned __int128)parts << 64) / v.nb);
+    const size_t smem = (size_t)kBulkChunk * (sizeof(Key) + (VIN ? sizeof(Val) : 0) + 2);
+    allow_smem(k_bulk_split<KIND, VIN>, smem);
+    k_bulk_split<KIND, VIN><<<chunks, kBulkThreads, smem, s>>>(v, (const Key *)keys, (const Val *)vals, n, parts,
+                                                               part_mul, sc);
+    // as many runs per warp as fill its keys without spilling into a second round
+    const long long want = (long long)R * 7 / 8 * parts / kBulkChunk;
+    const int runs = (int)std::max<long long>(1, std::min<long long>(want, kBulkRuns));
+    const int groups = (chunks + runs - 1) / runs;
+    const unsigned grid = (unsigned)(((long long)parts * groups * 32 + NT - 1) / NT);
+    k_bulk_probe<KIND, BB, OP, NT, R, MINB><<<grid, NT, 0, s>>>(v, sc, chunks, parts, groups, runs);
+    if (T::MAP && OP == OP_FIND && vals_out)
+        k_bulk_join<Key, Val, true><<<chunks, kBulkThreads, 0, s>>>(n, sc, out, (Val *)vals_out);
+    else if (out)
+        k_bulk_join<Key, Val, false><<<chunks, kBulkThreads, 0, s>>>(n, sc, out, nullptr);
+    return cudaGetLastError();
+}
+
+template <int KIND, int BB>
+cudaError_t launch_bulk_bb(int op, const View &v, const void *keys, const void *vals, long long n, uint8_t *out,
+                           void *vals_out, int parts, void *scratch, cudaStream_t s) {
+    switch (op) {
+        case OP_INSERT: return launch_bulk_op<KIND, BB, OP_INSERT>(v, keys, vals, n, out, nullptr, parts, scratch, s);
+        case OP_FIND: return launch_bulk_op<KIND, BB, OP_FIND>(v, keys, nullptr, n, out, vals_out, parts, scratch, s);
+        default: return launch_bulk_op<KIND, BB, OP_ERASE>(v, keys, nullptr, n, out, nullptr, parts, scratch, s);
+    }
+}
+
+// A bulk call on n keys of any number, piece after piece through one scratch.
+template <int KIND>
+cudaError_t launch_bulk(int op, const View &v, int bucket_bytes, const void *keys, const void *vals, long long n,
+                        uint8_t *out, void *vals_out, int parts, void *scratch, cudaStream_t s) {
+    using T = Traits<KIND>;
+    const auto *k = static_cast<const typename T::Key *>(keys);
+    const auto *val = static_cast<const typename T::Val *>(vals);
+    auto *vo = static_cast<typename T::Val *>(vals_out);
+    for (long long at = 0; at < n; at += kBulkPiece) {
+        const long long m = std::min<long long>(kBulkPiece, n - at);
+        const void *pk = k + at, *pv = val ? val + at : nullptr;
+        uint8_t *po = out ? out + at : nullptr;
+        void *pvo = vo ? vo + at : nullptr;
+        cudaError_t e;
+        switch (bucket_bytes) {
+            case 32: e = launch_bulk_bb<KIND, 32>(op, v, pk, pv, m, po, pvo, parts, scratch, s); break;
+            case 64: e = launch_bulk_bb<KIND, 64>(op, v, pk, pv, m, po, pvo, parts, scratch, s); break;
+            case 128: e = launch_bulk_bb<KIND, 128>(op, v, pk, pv, m, po, pvo, parts, scratch, s); break;
+            default: return cudaErrorInvalidValue;
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 template <int KIND, int BB>
 cudaError_t launch_clear_bb(const View &v, unsigned long long phys, unsigned long long capacity, int sm_count,
                             cudaStream_t s) {
@@ -331,6 +398,10 @@ cudaError_t launch_rehash(const View &old_v, unsigned long long old_phys, const 
                              uint8_t *out, void *vals_out, const LaunchShape &sh, const uint8_t *skip,              \
                              cudaStream_t s) {                                                                      \
         return launch_range<KIND>(op, v, bb, keys, vals, n, out, vals_out, sh, skip, s);                            \
+    }                                                                                                               \
+    cudaError_t NAME##_bulk(int op, const View &v, int bb, const void *keys, const void *vals, long long n,         \
+                            uint8_t *out, void *vals_out, int parts, void *scratch, cudaStream_t s) {               \
+        return launch_bulk<KIND>(op, v, bb, keys, vals, n, out, vals_out, parts, scratch, s);                       \
     }                                                                                                               \
     cudaError_t NAME##_clear(const View &v, unsigned long long phys, unsigned long long cap, int bb, int sms,       \
                              cudaStream_t s) {                                                                      \

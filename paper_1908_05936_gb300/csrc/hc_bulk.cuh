@@ -225,9 +225,9 @@ k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs
         upto[lane] = (int)incl > base ? incl - (unsigned)base : 0u;
         __syncwarp();
         RunsSrc<KIND> src{reinterpret_cast<const Key *>(sc.keys), reinterpret_cast<const Val *>(sc.vals), start, upto};
-        if constexpr (OP == OP_INSERT) insert_run<KIND, BB>(v, src, m, w.stack, w.st, cnts);
-        else if constexpr (OP == OP_FIND) find_run<KIND, BB>(v, src, m, w.stack, w.st, w.vals);
-        else erase_run<KIND, BB>(v, src, m, w.stack, w.st, cnts);
+        if constexpr (OP == OP_INSERT) insert_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
+        else if constexpr (OP == OP_FIND) find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals);
+        else erase_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
         for (int i = lane; i < m; i += 32) {
             const unsigned to = src.place(i);
             st_stream(sc.out + to, w.st[i]);

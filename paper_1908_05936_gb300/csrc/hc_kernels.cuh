@@ -193,8 +193,12 @@ void allow_smem(K kernel, size_t bytes) {
 // lose as much on erases).
 constexpr int kRunWarps = 48;
 
-template <int KIND, int BB, int OP, int R>
-cudaError_t launch_run(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
+// Tables from which lanes read wide buckets together (see_bucket; between 256
+// MB, where it costs 0-17 %, and 512 MB, where it gains 5-50 %).
+constexpr long long kTogetherBytes = 512ll << 20;
+
+template <int KIND, int BB, int OP, int R, bool TOGETHER>
+cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
                        const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     using T = Traits<KIND>;
     const long long even = (n + (long long)sh.sms * kRunWarps - 1) / ((long long)sh.sms * kRunWarps);
@@ -202,10 +206,20 @@ cudaError_t launch_run(const View &v, const void *keys, const void *vals, long l
     const long long per_block = (long long)(sh.block / 32) * run;
     const unsigned grid = (unsigned)((n + per_block - 1) / per_block);
     const size_t smem = sizeof(WarpRun<KIND, OP, R>) * (sh.block / 32);
-    allow_smem(k_run<KIND, BB, OP, R>, smem);
-    k_run<KIND, BB, OP, R><<<grid, sh.block, smem, s>>>(v, (const typename T::Key *)keys, (const typename T::Val *)vals,
+    allow_smem(k_run<KIND, BB, OP, R, TOGETHER>, smem);
+    k_run<KIND, BB, OP, R, TOGETHER><<<grid, sh.block, smem, s>>>(v, (const typename T::Key *)keys, (const typename T::Val *)vals,
                                                         skip, n, run, out, (typename T::Val *)vals_out);
     return cudaGetLastError();
+}
+
+template <int KIND, int BB, int OP, int R>
+cudaError_t launch_run(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
+                       const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
+    if constexpr (Slots<KIND, BB>::KRB > 32) {
+        if ((long long)v.nb * BB >= kTogetherBytes)
+            return launch_run_as<KIND, BB, OP, R, true>(v, keys, vals, n, out, vals_out, sh, skip, s);
+    }
+    return launch_run_as<KIND, BB, OP, R, false>(v, keys, vals, n, out, vals_out, sh, skip, s);
 }
 
 template <int KIND, int BB, int KPT, int S>
@@ -284,7 +298,8 @@ cudaError_t launch_range(int op, const View &v, int bucket_bytes, const void *ke
 }
 
 // The three passes of a bulk call on one piece of n <= kBulkPiece keys.  64
-// threads (two warps) per probing block: 24 blocks per SM hold 40 registers.
+// threads (two warps) per probing block: 24 blocks per SM hold 40 registers, 16
+// (wider key regions) 64.
 template <int KIND, int BB, int OP>
 cudaError_t launch_bulk_op(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
                            int parts, void *scratch, cudaStream_t s) {
@@ -292,7 +307,7 @@ cudaError_t launch_bulk_op(const View &v, const void *keys, const void *vals, lo
     using Key = typename T::Key;
     using Val = typename T::Val;
     constexpr bool VIN = T::MAP && OP == OP_INSERT;
-    constexpr int NT = 64, R = 256, MINB = 24;
+    constexpr int KRB = Slots<KIND, BB>::KRB, NT = 64, R = 256, MINB = KRB <= 32 ? 24 : 16;
     BulkScratch sc;
     bulk_scratch(&sc, static_cast<unsigned char *>(scratch), n, parts, (int)sizeof(Key), T::MAP ? (int)sizeof(Val) : 0, OP);
     const int chunks = (int)((n + kBulkChunk - 1) / kBulkChunk);

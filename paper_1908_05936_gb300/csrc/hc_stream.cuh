@@ -180,6 +180,88 @@ struct Drain {
     }
 };
 
+// What a key finds in a bucket, one bit per slot.
+struct Seen {
+    uint32_t hit, empty, tomb;
+};
+
+// Reads bucket b of every lane with `act` and compares it with the lane's key;
+// the whole warp calls it.  TOGETHER (key regions of 64 or 128 bytes): 2 or 4
+// lanes read a bucket together, one key of the group after another, so that a
+// bucket is one request however wide it is, and put their findings together;
+// otherwise a lane reads its own bucket, a request per 32 bytes.  Beyond the
+// reach of the address translation, where requests are what bounds a lookup,
+// the first wins; inside it the shuffles cost more than the requests.  set<u64>,
+// load factor 0.6, 2^22 present lookups, own -> together, G/s: 64-byte buckets
+// 1 GiB 26.4 -> 40.3, 512 MB 31.8 -> 41.7, 64 MB (2^20) 57 -> 47; 128-byte 1 GiB
+// 13.7 -> 23.8, 64 MB 34.8 -> 28.9; map<i64,i32>, 128-byte buckets (64 of keys):
+// 512 MB 20.8 -> 28.1, 256 MB (2^20, load factor 0.7) 29.9 -> 30.1, its inserts
+// 15.2 -> 13.1.
+template <int KIND, int BB, bool TOGETHER>
+__device__ __forceinline__ Seen see_bucket(const View &v, bool act, unsigned long long b,
+                                           typename Traits<KIND>::Key key) {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using Sl = Slots<KIND, BB>;
+    constexpr int SPB = Sl::SPB;
+    if constexpr (!TOGETHER || Sl::KRB <= 32) {
+        Seen m{0u, 0u, 0u};
+        if (act) {
+            LaneWords<Sl::KRB> lw;
+            lw.load(bucket_at<BB>(v, b));
+#pragma unroll
+            for (int x = 0; x < SPB; ++x) {
+                const Key ks = slot_key<KIND, Sl::KRB>(lw, x);
+                m.hit |= (uint32_t)(ks == key) << x;
+                m.empty |= (uint32_t)(ks == T::EMPTY) << x;
+                m.tomb |= (uint32_t)(ks == T::TOMB) << x;
+            }
+        }
+        return m;
+    } else {
+        constexpr int G = Sl::KRB / 32, PS = SPB / G;        // lanes per bucket, slots per lane
+        const int lane = threadIdx.x & 31, sub = lane & (G - 1), base = lane & ~(G - 1);
+        const unsigned acts = __ballot_sync(0xffffffffu, act);
+        LaneWords<32> lw[G];
+#pragma unroll
+        for (int r = 0; r < G; ++r) {
+            const unsigned long long rb = __shfl_sync(0xffffffffu, b, base + r);
+            if (acts >> (base + r) & 1u) lw[r].load(bucket_at<BB>(v, rb) + sub * 32);
+        }
+        Seen mine{0u, 0u, 0u};
+#pragma unroll
+        for (int r = 0; r < G; ++r) {
+            const Key rk = __shfl_sync(0xffffffffu, key, base + r);
+            Seen m{0u, 0u, 0u};
+            if (acts >> (base + r) & 1u) {
+#pragma unroll
+                for (int x = 0; x < PS; ++x) {
+                    const Key ks = slot_key<KIND, 32>(lw[r], x);
+                    m.hit |= (uint32_t)(ks == rk) << x;
+                    m.empty |= (uint32_t)(ks == T::EMPTY) << x;
+                    m.tomb |= (uint32_t)(ks == T::TOMB) << x;
+                }
+            }
+            if constexpr (SPB <= 8) {
+                uint32_t w = (m.hit | m.empty << 8 | m.tomb << 16) << (sub * PS);
+#pragma unroll
+                for (int d = 1; d < G; d <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, d);
+                m = Seen{w & 0xffu, w >> 8 & 0xffu, w >> 16};
+            } else {
+                m = Seen{m.hit << (sub * PS), m.empty << (sub * PS), m.tomb << (sub * PS)};
+#pragma unroll
+                for (int d = 1; d < G; d <<= 1) {
+                    m.hit |= __shfl_xor_sync(0xffffffffu, m.hit, d);
+                    m.empty |= __shfl_xor_sync(0xffffffffu, m.empty, d);
+                    m.tomb |= __shfl_xor_sync(0xffffffffu, m.tomb, d);
+                }
+            }
+            if (r == sub) mine = m;
+        }
+        return mine;
+    }
+}
+
 // Stack entries: the key, its next bucket << 16 | its position in the run, and
 // for inserts the value and the first free slot the key has passed (slot
 // position << 1 | was EMPTY; all ones: none).
@@ -196,14 +278,12 @@ struct Stack {
 
 // Looks up the keys src.key(i), i < cnt (asked for 32 at a time, in order, by
 // the whole warp); found flags go to sf[i], values to sv[i].
-template <int KIND, int BB, class Src>
+template <int KIND, int BB, bool TOGETHER, class Src>
 __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack<KIND, 1> &st, uint8_t *sf,
                                          typename Traits<KIND>::Val *sv) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
-    using Sl = Slots<KIND, BB>;
-    constexpr int LB = Sl::KRB;              // one thread reads the whole key region
     const int lane = threadIdx.x & 31;
     int next = 0, top = 0;
     Key ahead = lane < cnt ? src.key(lane) : Key();
@@ -243,31 +323,22 @@ __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack
             break;
         }
         __syncwarp();                        // entries are read before this step's survivors overwrite them
-        LaneWords<LB> lw;
-        if (act) load_find<LB>(lw, bucket_at<BB>(v, b));
+        const Seen seen = see_bucket<KIND, BB, TOGETHER>(v, act, b, key);
         if constexpr (T::MAP) {
             if (late >= 0) sv[late] = late_val;
             late = -1;
         }
         bool left = false;
         if (act) {
-            int hit = -1;
-            bool empty = false;
-#pragma unroll
-            for (int x = 0; x < Sl::SPB; ++x) {
-                const Key ks = slot_key<KIND, LB>(lw, x);
-                if (ks == key) hit = x;
-                empty |= ks == T::EMPTY;
-            }
-            if (hit >= 0) {
+            if (seen.hit) {
                 sf[idx] = 1;
                 if constexpr (T::MAP) {
                     late = idx;
-                    late_val = (Val)load_find_val<KIND, BB>(v, b, hit);
+                    late_val = (Val)load_val<KIND, BB>(v, b, __ffs(seen.hit) - 1);
                 }
             } else {
                 b = next_bucket(v, b);
-                left = !empty && !came_round(v, (unsigned long long)key, b, reach);
+                left = !seen.empty && !came_round(v, (unsigned long long)key, b, reach);
                 if (!left) {
                     sf[idx] = 0;
                     if constexpr (T::MAP) sv[idx] = (Val)0;
@@ -297,24 +368,13 @@ __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack
         __syncwarp();
         const int unread = d.unread(v, (unsigned long long)key, b, reach);
         const unsigned long long mine = Drain::bucket(v, b, d.sub);
-        int hit = -1;
-        bool empty = false;
-        if (act && d.sub < unread) {
-            LaneWords<LB> lw;
-            load_find<LB>(lw, bucket_at<BB>(v, mine));
-#pragma unroll
-            for (int x = 0; x < Sl::SPB; ++x) {
-                const Key ks = slot_key<KIND, LB>(lw, x);
-                if (ks == key) hit = x;
-                empty |= ks == T::EMPTY;
-            }
-        }
-        const unsigned stop = d.ballot(hit >= 0 || empty);
+        const Seen seen = see_bucket<KIND, BB, TOGETHER>(v, act && d.sub < unread, mine, key);
+        const unsigned stop = d.ballot(seen.hit || seen.empty);
         bool left = false;
         if (act && stop) {
             if (d.sub == __ffs(stop) - 1) {
-                sf[idx] = hit >= 0 ? 1 : 0;
-                if constexpr (T::MAP) sv[idx] = hit >= 0 ? (Val)load_find_val<KIND, BB>(v, mine, hit) : (Val)0;
+                sf[idx] = seen.hit ? 1 : 0;
+                if constexpr (T::MAP) sv[idx] = seen.hit ? (Val)load_val<KIND, BB>(v, mine, __ffs(seen.hit) - 1) : (Val)0;
             }
         } else if (act && d.sub == 0) {
             left = unread == d.group;
@@ -343,7 +403,7 @@ __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack
 // loses its slot to another key goes on from that slot's bucket: the buckets
 // before it had no free slot, and inserts never free one.  Equal keys inside a
 // warp are not folded here (folding is a lock-step option).
-template <int KIND, int BB, class Src>
+template <int KIND, int BB, bool TOGETHER, class Src>
 __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Stack<KIND, 0> &st, uint8_t *ss,
                                            Counts &cnts) {
     using T = Traits<KIND>;
@@ -443,24 +503,15 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
             break;
         }
         __syncwarp();                        // entries are read before this step's survivors overwrite them
-        LaneWords<LB> lw;
-        if (act) lw.load(bucket_at<BB>(v, b));
+        const Seen seen = see_bucket<KIND, BB, TOGETHER>(v, act, b, key);
+        const uint32_t le = seen.empty;
         bool left = false, claim = false;
         if (act) {
-            bool hit = false;
-            uint32_t le = 0, lt = 0;
-#pragma unroll
-            for (int x = 0; x < SPL; ++x) {
-                const Key ks = slot_key<KIND, LB>(lw, x);
-                hit |= ks == key;
-                le |= (uint32_t)(ks == T::EMPTY) << x;
-                lt |= (uint32_t)(ks == T::TOMB) << x;
-            }
-            if (hit) {                       // already stored
+            if (seen.hit) {                  // already stored
                 ss[idx] = (uint8_t)ST_EXISTS;
             } else {
                 if (at == NONE) {            // first free slot, rotated scan
-                    const uint32_t lf = le | (lt & claimable<KIND, BB, LB>(v, b, 0));
+                    const uint32_t lf = le | (seen.tomb & claimable<KIND, BB, LB>(v, b, 0));
                     if (lf) {
                         const int rot = v.rotate ? slot_rotation<Lay::SPB>((unsigned long long)key) : 0;
                         const uint32_t hi = lf & (Lay::ALL & ~((1u << rot) - 1u));
@@ -506,21 +557,11 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
         __syncwarp();
         const int unread = d.unread(v, (unsigned long long)key, b, reach);
         const unsigned long long mine = Drain::bucket(v, b, d.sub);
-        bool hit = false;
-        uint32_t le = 0;
+        const Seen seen = see_bucket<KIND, BB, TOGETHER>(v, act && d.sub < unread, mine, key);
+        const uint32_t le = seen.empty;
         unsigned long long here = NONE;                      // first free slot of this lane's bucket
-        if (act && d.sub < unread) {
-            LaneWords<LB> lw;
-            lw.load(bucket_at<BB>(v, mine));
-            uint32_t lt = 0;
-#pragma unroll
-            for (int x = 0; x < SPL; ++x) {
-                const Key ks = slot_key<KIND, LB>(lw, x);
-                hit |= ks == key;
-                le |= (uint32_t)(ks == T::EMPTY) << x;
-                lt |= (uint32_t)(ks == T::TOMB) << x;
-            }
-            const uint32_t lf = le | (lt & claimable<KIND, BB, LB>(v, mine, 0));
+        {
+            const uint32_t lf = le | (seen.tomb & claimable<KIND, BB, LB>(v, mine, 0));
             if (lf) {
                 const int rot = v.rotate ? slot_rotation<Lay::SPB>((unsigned long long)key) : 0;
                 const uint32_t hi = lf & (Lay::ALL & ~((1u << rot) - 1u));
@@ -528,8 +569,8 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
                 here = (mine * SPL + x) << 1 | (le >> x & 1u);
             }
         }
-        const unsigned stop = d.ballot(hit || le != 0);
-        const unsigned stored = d.ballot(hit);
+        const unsigned stop = d.ballot(seen.hit || le);
+        const unsigned stored = d.ballot(seen.hit != 0);
         const unsigned some = d.ballot(here != NONE);
         const unsigned first = stop & (0u - stop);           // the bucket that ends the probe, if any
         const unsigned upto = first ? (first - 1u) | first : 0xffffffffu;
@@ -574,13 +615,12 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
 // occurrences: NOT_FOUND); statuses go to ss[i].  A failed swap means an equal
 // key of the same call erased the slot first: that key reports ERASED, this one
 // NOT_FOUND.
-template <int KIND, int BB, class Src>
+template <int KIND, int BB, bool TOGETHER, class Src>
 __device__ __forceinline__ void erase_run(const View &v, Src &src, int cnt, Stack<KIND, 2> &st, uint8_t *ss,
                                           Counts &cnts) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Sl = Slots<KIND, BB>;
-    constexpr int LB = Sl::KRB;
     const int lane = threadIdx.x & 31;
     int next = 0, top = 0;
     Key ahead = Key();
@@ -629,26 +669,17 @@ __device__ __forceinline__ void erase_run(const View &v, Src &src, int cnt, Stac
             break;
         }
         __syncwarp();                        // entries are read before this step's survivors overwrite them
-        LaneWords<LB> lw;
-        if (act) lw.load(bucket_at<BB>(v, b));
+        const Seen seen = see_bucket<KIND, BB, TOGETHER>(v, act, b, key);
         bool left = false;
         if (act) {
-            int hit = -1;
-            bool empty = false;
-#pragma unroll
-            for (int x = 0; x < Sl::SPB; ++x) {
-                const Key ks = slot_key<KIND, LB>(lw, x);
-                if (ks == key) hit = x;
-                empty |= ks == T::EMPTY;
-            }
-            if (hit >= 0) {
-                const bool won = cas_key<KIND>(Sl::key(v, b, hit), key, T::TOMB) == key;
+            if (seen.hit) {
+                const bool won = cas_key<KIND>(Sl::key(v, b, __ffs(seen.hit) - 1), key, T::TOMB) == key;
                 if (won) note_claim_key<KIND>(v.hdr, key, -1);
                 ss[idx] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
                 cnts.del += won ? 1u : 0u;
             } else {
                 b = next_bucket(v, b);
-                left = !empty && !came_round(v, (unsigned long long)key, b, reach);
+                left = !seen.empty && !came_round(v, (unsigned long long)key, b, reach);
                 if (!left) ss[idx] = (uint8_t)ST_NOT_FOUND;
             }
         }
@@ -672,23 +703,12 @@ __device__ __forceinline__ void erase_run(const View &v, Src &src, int cnt, Stac
         __syncwarp();
         const int unread = d.unread(v, (unsigned long long)key, b, reach);
         const unsigned long long mine = Drain::bucket(v, b, d.sub);
-        int hit = -1;
-        bool empty = false;
-        if (act && d.sub < unread) {
-            LaneWords<LB> lw;
-            lw.load(bucket_at<BB>(v, mine));
-#pragma unroll
-            for (int x = 0; x < Sl::SPB; ++x) {
-                const Key ks = slot_key<KIND, LB>(lw, x);
-                if (ks == key) hit = x;
-                empty |= ks == T::EMPTY;
-            }
-        }
-        const unsigned stop = d.ballot(hit >= 0 || empty);
+        const Seen seen = see_bucket<KIND, BB, TOGETHER>(v, act && d.sub < unread, mine, key);
+        const unsigned stop = d.ballot(seen.hit || seen.empty);
         bool left = false;
         if (act && stop) {
             if (d.sub == __ffs(stop) - 1) {
-                const bool won = hit >= 0 && cas_key<KIND>(Sl::key(v, mine, hit), key, T::TOMB) == key;
+                const bool won = seen.hit && cas_key<KIND>(Sl::key(v, mine, __ffs(seen.hit) - 1), key, T::TOMB) == key;
                 if (won) note_claim_key<KIND>(v.hdr, key, -1);
                 ss[idx] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
                 cnts.del += won ? 1u : 0u;
@@ -770,12 +790,17 @@ struct BlockCounts {
     }
 };
 
+// Blocks of 256 threads per SM that the probe loops are compiled for, by the
+// key region that a key in flight holds in registers: 5 (51 registers) for 32
+// bytes (at 6, 40 registers and 20-40 bytes spilled, lookups and inserts beyond
+// L2 are 2-6 % slower, at 8, 32 registers, 10-20 %), 4 (64) for wider ones, 3
+// where 128 bytes are read by lanes together.
+constexpr int run_blocks(int krb, bool together) { return krb <= 32 ? 5 : krb == 128 && together ? 3 : 4; }
+
 // The range kernels: warp w of the grid takes keys [w * run, w * run + run),
-// run <= R.  5 blocks of 256 threads (51 registers) keep every kind's state
-// without spills; at 6 (40 registers, 20-40 bytes spilled) lookups and inserts
-// beyond L2 are 2-6 % slower, at 8 (32) 10-20 %.
-template <int KIND, int BB, int OP, int R>
-__global__ void __launch_bounds__(256, 5)
+// run <= R.
+template <int KIND, int BB, int OP, int R, bool TOGETHER>
+__global__ void __launch_bounds__(256, run_blocks(Slots<KIND, BB>::KRB, TOGETHER))
 k_run(View v, const typename Traits<KIND>::Key *keys, const typename Traits<KIND>::Val *vals, const uint8_t *skip,
       long long n, int run, uint8_t *out, typename Traits<KIND>::Val *vals_out) {
     using T = Traits<KIND>;
@@ -790,9 +815,9 @@ k_run(View v, const typename Traits<KIND>::Key *keys, const typename Traits<KIND
     debug_range(v, c0, cnt, n);
     ArraySrc<KIND> src{keys + c0, vals + c0, skip ? skip + c0 : nullptr};
     Counts cnts;
-    if constexpr (OP == 0) insert_run<KIND, BB>(v, src, cnt, w.stack, w.st, cnts);
-    else if constexpr (OP == 1) find_run<KIND, BB>(v, src, cnt, w.stack, w.st, w.vals);
-    else erase_run<KIND, BB>(v, src, cnt, w.stack, w.st, cnts);
+    if constexpr (OP == 0) insert_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, cnts);
+    else if constexpr (OP == 1) find_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, w.vals);
+    else erase_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, cnts);
     for (int i = threadIdx.x & 31; i < cnt; i += 32) {
         if (out) st_stream(out + c0 + i, w.st[i]);
         if constexpr (OP == 1 && T::MAP) {

@@ -274,7 +274,6 @@ __global__ void k_set_u64(unsigned long long *p, unsigned long long v) { *p = v;
 
 __global__ void k_rehash_finish(hc::Header *old_h, hc::Header *new_h) {
     new_h->live = old_h->live;
-    new_h->used = new_h->reinserted;
     new_h->err |= old_h->err;
     new_h->side_present[0] = old_h->side_present[0];
     new_h->side_present[1] = old_h->side_present[1];
@@ -690,8 +689,7 @@ hc_rc hc_dump(hc_table *t, void *d_keys_out, void *d_vals_out, int64_t cap, int6
     fill_view(t, &dv);
     const hc::SelectPred all{HC_PRED_ALL, 0, 0, 0, {}};
     const cudaError_t e = hc::select_entries(dv, all, d_keys_out, is_map(t->kind) ? d_vals_out : nullptr,
-                                             (unsigned long long)cap, &t->view.hdr->dump_count,
-                                             (unsigned long long)t->phys + 2ull, sm_count_of(t->device), s);
+                                             (unsigned long long)cap, &t->view.hdr->dump_count, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the dump kernel");
     hc::Header h;
     if ((rc = read_header(t, &h, s)) != HC_OK) return rc;
@@ -779,7 +777,6 @@ hc_rc hc_select(hc_table *t, const hc_predicate *pred, void *d_keys_out, void *d
     for (int i = 0; i < 6; ++i) p.box[i] = pred->box[i];
     const cudaError_t e = hc::select_entries(dv, p, d_keys_out, is_map(t->kind) ? d_vals_out : nullptr,
                                              (unsigned long long)cap, reinterpret_cast<unsigned long long *>(d_count),
-                                             (unsigned long long)t->phys + 2ull, sm_count_of(t->device),
                                              static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "launching the selection kernel");
     return HC_OK;

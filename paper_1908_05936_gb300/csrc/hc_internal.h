@@ -108,6 +108,6 @@ cudaError_t unpack_short3(const long long *keys, long long n, int16_t *xyz, int 
 
 // Appends the stored entries of the table behind dv that satisfy p (hc_select).
 cudaError_t select_entries(const hc_device_view &dv, const SelectPred &p, void *ko, void *vo, unsigned long long cap,
-                           unsigned long long *count, unsigned long long positions, int sms, cudaStream_t s);
+                           unsigned long long *count, cudaStream_t s);
 
 }  // namespace hc

@@ -115,18 +115,18 @@ typedef struct hc_config {
  * key); each group handles keys_per_group keys at once so that several
  * bucket reads are in flight per lane.  Zero fields keep the current value.
  * keys_per_group 4 or 8 (any operation, lane_bytes = the key region)
- * selects the streaming form: a block stages its keys in shared memory and
- * each thread keeps 2 or 4 probes in flight, refilling as they finish (no
- * duplicate folding in this form).  Defaults:
- * lane_bytes = the bucket's key region (one thread per key),
- * keys_per_group 4 (streaming), block 64, folding off; until hc_set_launch
- * sets an op's shape, a plain insert of fewer than 8192 keys per
- * multiprocessor and at most one key per bucket, into a table whose buckets
- * exceed the L2 cache, runs one key per thread in lock step.  Results never
- * depend on the shape. */
+ * selects warp runs: a warp works through up to 128 or 256 keys, keeping those
+ * that need more than one bucket on a stack (no duplicate folding in this
+ * form).  Defaults:
+ * lane_bytes = the bucket's key region, keys_per_group 4 (warp runs), block
+ * 128, folding off; until hc_set_launch sets an op's shape, a large hc_insert,
+ * hc_find or hc_erase on a table of 512 MB or more may run as three passes over
+ * stream-ordered scratch of its own (11 to 19 bytes a key, for at most 2^26 keys
+ * at a time; a capturing stream, or memory that is not there, keeps the range
+ * kernel).  Results never depend on the shape. */
 typedef struct hc_launch {
     int32_t lane_bytes;       /* 32, 64 or 128, at most bucket_bytes     */
-    int32_t keys_per_group;   /* 1 or 2; 4 or 8: streaming forms       */
+    int32_t keys_per_group;   /* 1 or 2; 4 or 8: warp runs             */
     int32_t block;            /* threads per block: 64..256, multiple of 32  */
     int32_t fold_duplicates;  /* 1: equal keys inside a warp are folded to
                                  one probe (__match_any_sync); 2: off      */
@@ -417,14 +417,16 @@ typedef struct hc_batch_item {
 
 typedef struct hc_batch_config {
     int32_t lane_bytes;      /* 0: one thread per key (whole bucket); 32: 32-byte lanes */
-    int32_t keys_per_group;  /* 1 or 2: lock-step phases (default 1); 4 or 8:
-                                streaming phases (keys staged per block, 2 or
-                                4 probes in flight per thread; block <= 256) */
-    int32_t block;           /* threads per block (0 = 256)                */
-    int32_t blocks_per_sm;   /* persistent grid = SMs x this (0 = auto)    */
+    int32_t keys_per_group;  /* 1 or 2: lock-step phases; 4 or 8: warp runs of
+                                up to 128 or 256 keys (0 = 8)              */
+    int32_t block;           /* threads per block (0 = 64 for warp runs, 256
+                                for lock-step phases)                      */
+    int32_t blocks_per_sm;   /* persistent grid = SMs x this (0: one warp per
+                                chunk)                                     */
     int32_t tile;            /* keys per chunk, a multiple of 128 (0 = auto:
-                                128..1024 from the total keys, so that the
-                                chunks can occupy every warp slot)          */
+                                from the total keys, so that the chunks can
+                                occupy every warp slot: 128..256 for warp
+                                runs, 128..1024 for lock-step phases)       */
     int32_t use_graph;       /* 1: capture the three phases in a CUDA graph */
 } hc_batch_config;
 

@@ -2,13 +2,13 @@
 // persistent launch per phase (insert, then find, then erase), optionally
 // captured once into a CUDA graph and replayed.
 //
-// Scheduling.  Every item is cut into chunks of `tile` keys.  A phase kernel
-// runs a persistent grid (SMs x blocks per SM); each warp takes the next
-// chunk number from a counter in global memory with one atomic add, finds the
-// item that chunk belongs to by binary search over the items' chunk offsets,
-// and runs the same warp-tile code as the one-launch-per-call kernels over
-// the chunk.  Tables of very different sizes are therefore balanced at chunk
-// granularity, and no launch is spent per table.
+// Scheduling.  Every item is cut into chunks of `tile` keys.  A phase kernel has
+// one warp per chunk (or, with blocks_per_sm, a persistent grid whose warps
+// stride over the chunks); a warp finds the item its chunk belongs to by a
+// 32-way search over the items' chunk offsets and runs the same loops as the
+// one-launch-per-call kernels over the chunk.  Tables of very different sizes
+// are therefore balanced at chunk granularity, and no launch is spent per table.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -43,7 +43,6 @@ struct PhaseDesc {
     int item0;
     int n_items;
     long long n_chunks;
-    int counter;   // index of this phase's chunk counter
 };
 
 template <int KIND, int OP, int BB, int LB, int KPT>
@@ -58,64 +57,61 @@ __device__ __forceinline__ void run_chunk(const BatchItemDev &it, long long k0, 
     if constexpr (OP != OP_FIND) flush_counts(it.v, cnt);
 }
 
+// The item that chunk c of a phase belongs to: the last one whose chunk_begin
+// is at most c.  The whole warp calls it.
+__device__ __forceinline__ int item_of(const BatchItemDev *items, int n_items, long long c) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = n_items;
+    while (n > 1) {
+        const int step = (n + 31) / 32, at = lane * step;
+        const unsigned m = __ballot_sync(0xffffffffu, at < n && items[lo + (at < n ? at : 0)].chunk_begin <= c);
+        const int k = (__popc(m) - 1) * step;              // chunk_begin ascends: m is a run of low bits
+        lo += k;
+        n = n - k < step ? n - k : step;
+    }
+    return lo;
+}
+
 // One phase launch covers items of one kind, one op and one bucket size (so
 // each launch is a small specialisation).  WIDE: one thread per key reading
 // the whole bucket (maps: keys and values) or key region (sets); otherwise
 // 32-byte lanes.
 template <int KIND, int OP, int BB, int WIDE, int KPT>
 __global__ void __launch_bounds__(256)
-k_batch_phase(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile,
-              unsigned long long *counter) {
+k_batch_phase(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile) {
     constexpr int KRB = Slots<KIND, BB>::KRB;
     constexpr int LB = WIDE ? (Traits<KIND>::MAP ? BB : KRB) : (KRB < 32 ? KRB : 32);
-    const int lane = threadIdx.x & 31;
-    while (true) {
-        unsigned long long c = 0;
-        if (lane == 0) c = atomicAdd(counter, 1ull);
-        c = __shfl_sync(0xffffffffu, c, 0);
-        if ((long long)c >= n_chunks) break;
-        // last item whose chunk_begin <= c
-        int lo = 0, hi = n_items - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (items[mid].chunk_begin <= (long long)c) lo = mid;
-            else hi = mid - 1;
-        }
-        const BatchItemDev it = items[lo];
-        const long long k0 = ((long long)c - it.chunk_begin) * tile;
+    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_chunks; c += warps) {
+        const BatchItemDev it = items[item_of(items, n_items, c)];
+        const long long k0 = (c - it.chunk_begin) * tile;
         const long long k1 = k0 + tile < it.n ? k0 + tile : it.n;
         debug_range(it.v, k0, k1 - k0, it.n);
         run_chunk<KIND, OP, BB, LB, KPT>(it, k0, k1);
     }
 }
 
-// The warp-run form of a phase (keys_per_group 4 or 8): a warp takes the next
-// chunk with one atomic add and works through it in runs of up to R keys with
-// the range kernels' probe loops.
+// The warp-run form of a phase (keys_per_group 4 or 8, the default): a warp
+// works through its chunk in runs of up to R keys with the range kernels' probe
+// loops.  Inserts and erases run at the rate at which a compare-and-swap follows
+// a read of the same line inside L2 (50 G/s; the tables of the chunks in flight
+// are there), lookups at 60 % of the copy peak.  Against lock-step phases whose
+// warps took chunks from one counter: 192 set<u64> of 2^10-2^20 slots, 25 M
+// operations, 750 -> 547 us; 1024 tables, 127 M operations, 3.21 -> 2.50 ms.
 template <int KIND, int OP, int BB, int R>
 __global__ void __launch_bounds__(256, 5)
-k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile,
-            unsigned long long *counter) {
+k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
     extern __shared__ __align__(16) unsigned char smem[];
     WarpRun<KIND, OP, R> &w = reinterpret_cast<WarpRun<KIND, OP, R> *>(smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    while (true) {
-        unsigned long long c = 0;
-        if (lane == 0) c = atomicAdd(counter, 1ull);
-        c = __shfl_sync(0xffffffffu, c, 0);
-        if ((long long)c >= n_chunks) break;
-        int lo = 0, hi = n_items - 1;                      // last item whose chunk_begin <= c
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (items[mid].chunk_begin <= (long long)c) lo = mid;
-            else hi = mid - 1;
-        }
-        const BatchItemDev &it = items[lo];
+    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_chunks; c += warps) {
+        const BatchItemDev &it = items[item_of(items, n_items, c)];
         const View v = it.v;
-        const long long k0 = ((long long)c - it.chunk_begin) * tile;
+        const long long k0 = (c - it.chunk_begin) * tile;
         const long long k1 = k0 + tile < it.n ? k0 + tile : it.n;
         Counts cnts;
         for (long long p0 = k0; p0 < k1; p0 += R) {
@@ -137,11 +133,7 @@ k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chu
     }
 }
 
-__global__ void k_zero_counters(unsigned long long *c, int n) {
-    if (threadIdx.x < n) c[threadIdx.x] = 0ull;
-}
-
-using PhaseKernel = void (*)(const BatchItemDev *, int, long long, int, unsigned long long *);
+using PhaseKernel = void (*)(const BatchItemDev *, int, long long, int);
 
 template <int KIND, int OP, int BB>
 PhaseKernel pick_lb_kpt(int lb, int kpt) {
@@ -202,9 +194,8 @@ struct hc_batch {
     int device;
     int block, blocks_per_sm, tile, lane_bytes, kpt;
     bool use_graph;
-    void *d_mem = nullptr;   // items then counters
+    void *d_mem = nullptr;
     hc::BatchItemDev *d_items = nullptr;
-    unsigned long long *d_counters = nullptr;
     std::vector<hc::PhaseDesc> phases;
     std::vector<int> grid;
     cudaGraph_t graph = nullptr;
@@ -220,21 +211,23 @@ namespace {
 constexpr uint32_t kBatchMagic = 0x48434241u;
 
 // tile 0 in the configuration: keys per chunk chosen from the total work so
-// that the chunks can occupy every warp slot of the GPU (64 per SM): a power
-// of two from 128 to 4096.
-int auto_tile(const hc_batch_item *items, int64_t n_items) {
+// that the chunks can occupy every warp slot of the GPU (64 per SM): a power of
+// two from 128 to 1024, to 256 for warp runs (192 set<u64> of 2^10-2^20 slots,
+// 25 M operations, with chunks of 128, 256, 512, 1024: 554, 547, 578, 609 us).
+int auto_tile(const hc_batch_item *items, int64_t n_items, int kpt) {
+    const int most = kpt >= 4 ? 256 : 1024;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                    cudaSuccess || sms <= 0) {
         (void)cudaGetLastError();
-        return 4096;
+        return most;
     }
     long long total = 0;
     for (int64_t i = 0; i < n_items; ++i)
         if (items[i].n > 0) total += items[i].n;
     const long long per_slot = total / ((long long)sms * 64);
     int tile = 128;
-    while (tile < 1024 && (long long)tile * 2 <= per_slot) tile *= 2;
+    while (tile < most && (long long)tile * 2 <= per_slot) tile *= 2;
     return tile;
 }
 
@@ -244,20 +237,21 @@ hc_rc bcuda(cudaError_t e, const char *what) {
     return bfail(HC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// Blocks of a phase: one warp per chunk, or a persistent grid of per_sm blocks
+// per SM where the configuration asks for one.
+unsigned phase_grid(const hc::PhaseDesc &ph, int block, int per_sm, int sms) {
+    const long long need = (ph.n_chunks * 32 + block - 1) / block;
+    return (unsigned)(per_sm > 0 ? std::min<long long>(need, (long long)sms * per_sm) : need);
+}
+
 hc_rc enqueue(hc_batch *b, cudaStream_t s) {
-    const int n_ctr = (int)b->phases.size();
-    if (n_ctr == 0) return HC_OK;
-    hc::k_zero_counters<<<1, 64, 0, s>>>(b->d_counters, n_ctr);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return bcuda(e, "resetting the batch counters");
     for (size_t p = 0; p < b->phases.size(); ++p) {
         const hc::PhaseDesc &ph = b->phases[p];
         hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, b->lane_bytes, b->kpt);
         const size_t smem = hc::phase_smem(ph.kind, ph.op, b->kpt, b->block);
         hc::allow_phase_smem(k, smem);
-        k<<<b->grid[p], b->block, smem, s>>>(
-            b->d_items + ph.item0, ph.n_items, ph.n_chunks, b->tile, b->d_counters + ph.counter);
-        e = cudaGetLastError();
+        k<<<b->grid[p], b->block, smem, s>>>(b->d_items + ph.item0, ph.n_items, ph.n_chunks, b->tile);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return bcuda(e, "launching a batch phase");
     }
     return HC_OK;
@@ -275,9 +269,9 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     hc_batch_config c{};
     if (cfg) c = *cfg;
     const int lb = c.lane_bytes;
-    const int kpt = c.keys_per_group ? c.keys_per_group : 1;
-    const int block = c.block ? c.block : 256;
-    const int tile = c.tile ? c.tile : auto_tile(items, n_items);
+    const int kpt = c.keys_per_group ? c.keys_per_group : 8;
+    const int block = c.block ? c.block : kpt >= 4 ? 64 : 256;
+    const int tile = c.tile ? c.tile : auto_tile(items, n_items, kpt);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
         return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
@@ -291,7 +285,7 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     for (int op = 0; op < 3; ++op) {
         for (int kind = 0; kind < 4; ++kind)
         for (int bb = 32; bb <= 128; bb *= 2) {
-            hc::PhaseDesc ph{kind, op, bb, (int)dev.size(), 0, 0, (int)phases.size()};
+            hc::PhaseDesc ph{kind, op, bb, (int)dev.size(), 0, 0};
             for (int64_t i = 0; i < n_items; ++i) {
                 const hc_batch_item &it = items[i];
                 if (!it.table || it.table->magic != HC_TABLE_MAGIC) return bfail(HC_ERR_ARG, "item with a bad table");
@@ -333,35 +327,19 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     b->phases = phases;
     cudaError_t e = cudaGetDevice(&b->device);
     const size_t items_bytes = (dev.size() * sizeof(hc::BatchItemDev) + 255) / 256 * 256;
-    const size_t bytes = items_bytes + 512;   // up to 36 phase counters
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_mem, bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_mem, std::max<size_t>(items_bytes, 256));
     if (e != cudaSuccess) {
         delete b;
         return bcuda(e, "allocating the batch descriptors");
     }
     b->d_items = static_cast<hc::BatchItemDev *>(b->d_mem);
-    b->d_counters = reinterpret_cast<unsigned long long *>(static_cast<char *>(b->d_mem) + items_bytes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!dev.empty())
         e = cudaMemcpyAsync(b->d_items, dev.data(), dev.size() * sizeof(hc::BatchItemDev), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     int sms = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-    for (size_t p = 0; p < phases.size() && e == cudaSuccess; ++p) {
-        int per_sm = c.blocks_per_sm;
-        if (per_sm <= 0) {
-            hc::PhaseKernel k = hc::pick_kernel(phases[p].kind, phases[p].op, phases[p].bb, lb, kpt);
-            const size_t smem = hc::phase_smem(phases[p].kind, phases[p].op, kpt, block);
-            hc::allow_phase_smem(k, smem);
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
-            if (per_sm <= 0) per_sm = 1;
-        }
-        long long g = (long long)sms * per_sm;
-        // one warp per chunk at most
-        const long long need = (phases[p].n_chunks * 32 + block - 1) / block;
-        if (g > need) g = need;
-        b->grid.push_back((int)(g > 0 ? g : 1));
-    }
+    for (const hc::PhaseDesc &ph : phases) b->grid.push_back(phase_grid(ph, block, c.blocks_per_sm, sms));
     if (e == cudaSuccess && b->use_graph) {
         // capture on a private stream so the caller's stream is never in capture mode
         cudaStream_t cs;
@@ -414,8 +392,7 @@ HC_API hc_rc hc_batch_destroy(hc_batch *b) {
 }  // extern "C"
 
 // ---- batched form without any device allocation --------------------------
-// hc_batch_create allocates its item descriptors and chunk counters with
-// cudaMalloc.  This variant keeps them in one file-scope device array instead,
+// hc_batch_create allocates its item descriptors with cudaMalloc.  This variant keeps them in one file-scope device array instead,
 // for callers that must not allocate device memory themselves.  The array is
 // part of the library image: every GPU that loads the library holds it until
 // the process exits, and every call shares it.
@@ -427,7 +404,6 @@ constexpr int kNoAllocMaxPhases = 36;    // 3 operations x 4 container kinds x 3
 
 struct NoAllocScratch {
     hc::BatchItemDev items[kNoAllocMaxItems];
-    unsigned long long counters[64];
 };
 
 }  // namespace
@@ -473,9 +449,9 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     hc_batch_config c{};
     if (cfg) c = *cfg;
     const int lb = c.lane_bytes;
-    const int kpt = c.keys_per_group ? c.keys_per_group : 1;
-    const int block = c.block ? c.block : 256;
-    const int tile = c.tile ? c.tile : auto_tile(items, n_items);
+    const int kpt = c.keys_per_group ? c.keys_per_group : 8;
+    const int block = c.block ? c.block : kpt >= 4 ? 64 : 256;
+    const int tile = c.tile ? c.tile : auto_tile(items, n_items, kpt);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
         return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
@@ -490,7 +466,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     for (int op = 0; op < 3; ++op) {
         for (int kind = 0; kind < 4; ++kind)
         for (int bb = 32; bb <= 128; bb *= 2) {
-            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0, n_phases};
+            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0};
             for (int64_t i = 0; i < n_items; ++i) {
                 const hc_batch_item &it = items[i];
                 if (!it.table || it.table->magic != HC_TABLE_MAGIC) return bfail(HC_ERR_ARG, "item with a bad table");
@@ -539,26 +515,13 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     e = cudaMemcpyAsync(scratch->items, t_noalloc_items, (size_t)n_dev * sizeof(hc::BatchItemDev),
                         cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bcuda(e, "copying the batch descriptors");
-    // the chunk counters keep the previous call's values: reset them first
-    hc::k_zero_counters<<<1, 64, 0, s>>>(scratch->counters, n_phases);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return bcuda(e, "resetting the chunk counters");
     for (int p = 0; p < n_phases; ++p) {
         const hc::PhaseDesc &ph = phases[p];
         hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lb, kpt);
         const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
         hc::allow_phase_smem(k, smem);
-        int per_sm = c.blocks_per_sm;
-        if (per_sm <= 0) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
-            if (e != cudaSuccess) return bcuda(e, "querying occupancy");
-            if (per_sm <= 0) per_sm = 1;
-        }
-        long long g = (long long)sms * per_sm;
-        const long long need = (ph.n_chunks * 32 + block - 1) / block;
-        if (g > need) g = need;
-        k<<<(unsigned)(g > 0 ? g : 1), block, smem, s>>>(
-            scratch->items + ph.item0, ph.n_items, ph.n_chunks, tile, scratch->counters + ph.counter);
+        k<<<phase_grid(ph, block, c.blocks_per_sm, sms), block, smem, s>>>(scratch->items + ph.item0, ph.n_items,
+                                                                            ph.n_chunks, tile);
         e = cudaGetLastError();
         if (e != cudaSuccess) return bcuda(e, "launching a batch phase");
     }
@@ -571,7 +534,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
 // The served form forms a new batch at every dispatch.  Building a graph or
 // allocating descriptors per dispatch would cost more than small requests
 // themselves, so the caller hands in a device scratch buffer (one per stream
-// it dispatches on) that receives the descriptors and chunk counters.
+// it dispatches on) that receives the descriptors.
 
 namespace {
 
@@ -584,7 +547,7 @@ extern "C" {
 
 HC_API int64_t hc_batch_scratch_bytes(int64_t n_items) {
     if (n_items < 0 || n_items > kRunMaxItems) return -1;
-    return (int64_t)((n_items * sizeof(hc::BatchItemDev) + 255) / 256 * 256 + 512);   // + 36 counters
+    return (int64_t)((n_items * sizeof(hc::BatchItemDev) + 255) / 256 * 256 + 512);   // the last 512 bytes are spare
 }
 
 namespace {
@@ -612,9 +575,9 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     hc_batch_config c{};
     if (cfg) c = *cfg;
     const int lb = c.lane_bytes;
-    const int kpt = c.keys_per_group ? c.keys_per_group : 1;
-    const int block = c.block ? c.block : 256;
-    const int tile = c.tile ? c.tile : auto_tile(items, n_items);
+    const int kpt = c.keys_per_group ? c.keys_per_group : 8;
+    const int block = c.block ? c.block : kpt >= 4 ? 64 : 256;
+    const int tile = c.tile ? c.tile : auto_tile(items, n_items, kpt);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole key region) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
         return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
@@ -628,7 +591,7 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     for (int op = 0; op < 3; ++op) {
         for (int kind = 0; kind < 4; ++kind)
         for (int bb = 32; bb <= 128; bb *= 2) {
-            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0, n_phases};
+            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0};
             for (int64_t i = 0; i < n_items; ++i) {
                 const hc_batch_item &it = items[i];
                 if (!it.table || it.table->magic != HC_TABLE_MAGIC) return bfail(HC_ERR_ARG, "item with a bad table");
@@ -665,24 +628,16 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return bcuda(e, "reading the device");
     auto *d_items = static_cast<hc::BatchItemDev *>(d_scratch);
-    auto *d_ctr = reinterpret_cast<unsigned long long *>(static_cast<char *>(d_scratch) + need - 512);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     e = cudaMemcpyAsync(d_items, desc, (size_t)n_dev * sizeof(hc::BatchItemDev), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bcuda(e, "copying the batch descriptors");
-    hc::k_zero_counters<<<1, 64, 0, s>>>(d_ctr, n_phases);
     for (int p = 0; p < n_phases; ++p) {
         const hc::PhaseDesc &ph = phases[p];
         hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lb, kpt);
-        int per_sm = c.blocks_per_sm;
         const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
         hc::allow_phase_smem(k, smem);
-        if (per_sm <= 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem) != cudaSuccess) per_sm = 1;
-        if (per_sm <= 0) per_sm = 1;
-        long long g = (long long)sms * per_sm;
-        const long long want = (ph.n_chunks * 32 + block - 1) / block;
-        if (g > want) g = want;
-        k<<<(unsigned)(g > 0 ? g : 1), block, smem, s>>>(d_items + ph.item0, ph.n_items, ph.n_chunks, tile,
-                                                         d_ctr + ph.counter);
+        k<<<phase_grid(ph, block, c.blocks_per_sm, sms), block, smem, s>>>(d_items + ph.item0, ph.n_items, ph.n_chunks,
+                                                                            tile);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return bcuda(e, "launching the batch phases");

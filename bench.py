@@ -329,7 +329,7 @@ def run_gpu(args, rank: int, world: int):
     dom_ms = summary[dom]["ms_total"] / len(per[dom])
     achieved = BYTES_PER_OP[kinds[dom]] * dom_n / (dom_ms * 1e-3) / 1e9
     traffic = None
-    if (dom == "insert" and not in_kernel and bb == 64 and t.get_launch(0)["keys_per_group"] == 4
+    if (dom == "insert" and not in_kernel and bb == 64 and t.get_launch(0)["keys_per_group"] == 8
             and t.get_launch(0)["block"] == 128 and insert_kernel_digest() == INSERT_TRAFFIC["digest"]):
         traffic = INSERT_TRAFFIC["bytes_per_op"] * dom_n      # DRAM bytes per launch
     peak, peak_src = hbm_peak()

@@ -118,7 +118,7 @@ typedef struct hc_config {
  * selects warp runs: a warp works through up to 128 or 256 keys, keeping those
  * that need more than one bucket on a stack (no duplicate folding in this
  * form).  Defaults:
- * lane_bytes = the bucket's key region, keys_per_group 4 (warp runs), block
+ * lane_bytes = the bucket's key region, keys_per_group 8 (warp runs), block
  * 128, folding off; until hc_set_launch sets an op's shape, a large hc_insert,
  * hc_find or hc_erase on a table of 512 MB or more may run as three passes over
  * stream-ordered scratch of its own (11 to 19 bytes a key, for at most 2^26 keys

@@ -471,8 +471,8 @@ hc_rc hc_create(hc_table **out, int32_t kind, int64_t slots, const hc_config *cf
         return fail(HC_ERR_OOM, "cudaMalloc of %lld bytes failed: %s", (long long)g.bytes, cudaGetErrorString(e));
     }
     t->view = make_view(t->d_mem, g, seed, hm);
-    // the warp-run kernels with runs of up to 128 keys, 128-thread blocks
-    for (int op = 0; op < 3; ++op) t->shape[op] = hc::LaunchShape{key_region_bytes(kind, bb), 4, 128, 0, 0};
+    // the warp-run kernels with runs of up to 256 keys, 128-thread blocks
+    for (int op = 0; op < 3; ++op) t->shape[op] = hc::LaunchShape{key_region_bytes(kind, bb), 8, 128, 0, 0};
     e = dispatch_clear(t, t->view, t->phys, t->capacity, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
         cudaFree(t->d_mem);
@@ -745,7 +745,7 @@ hc_rc hc_erase_ordered(hc_table *t, const void *d_keys, int64_t n, uint8_t *d_st
     cudaError_t e = hc::ordered_leaders(d_keys, key_bytes(t->kind), n, d_scratch, &t->view.hdr->err, sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "finding the first occurrences");
     // the warp-run erase takes the skip flags (later occurrences: NOT_FOUND)
-    hc::LaunchShape sh{key_region_bytes(t->kind, t->bucket_bytes), 4, 128, 0, sms};
+    hc::LaunchShape sh{key_region_bytes(t->kind, t->bucket_bytes), 8, 128, 0, sms};
     e = dispatch_range(t->kind, hc::OP_ERASE, t->view, t->bucket_bytes, d_keys, nullptr, n, d_status, nullptr, sh,
                        hc::ordered_skip(n, d_scratch), s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the erase kernel");

@@ -181,24 +181,33 @@ void allow_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024) (void)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// The warp-run kernels (keys_per_group 4 or 8): runs of up to R = 128 or 256
-// keys per warp, shorter where n is too small to give every SM kRunWarps warps
-// (2^20 keys on a 1 GiB map, runs of 128 against 256: present lookups 19.1 and
-// 17.8 G/s, absent 16.6 and 14.6, inserts 9.5 and 8.4; from 2^24 keys on the
-// two are within 3 %, and runs of 64 gain 2-5 % on lookups and inserts but
-// lose as much on erases).
-constexpr int kRunWarps = 48;
+// Tables from which on the reach of the address translation is what matters.
+constexpr long long kBeyondReach = 512ll << 20;
+
+// The warp-run kernels (keys_per_group 4 or 8), the length of a run: what makes
+// one wave of equal runs of the warps that are resident together, if that is at
+// most R keys and the table is within reach (an RGB-D frame of 400,000
+// candidates 67 us with runs that fill 1.03 waves, 61 with one wave; the
+// L2-resident set<u32> workload 64 and 59); 128 for larger calls.  Beyond reach
+// shorter runs spread the wait for requests better (10^6 keys on an 800 MB map:
+// insert + lookup + erase 264 us in one wave of 192, 237 with 128, 233 with 64;
+// erases of 2^22 keys and more prefer 128 by 4 %).
+inline int run_length(int op, long long n, long long resident, int most, bool beyond) {
+    const long long wave = (n + resident * 32 - 1) / (resident * 32) * 32;
+    if (beyond) return (int)std::min<long long>(wave, op == OP_ERASE ? 128 : 64);
+    return wave <= most ? (int)wave : 128;
+}
 
 // Tables from which lanes read wide buckets together (see_bucket; between 256
 // MB, where it costs 0-17 %, and 512 MB, where it gains 5-50 %).
-constexpr long long kTogetherBytes = 512ll << 20;
+constexpr long long kTogetherBytes = kBeyondReach;
 
 template <int KIND, int BB, int OP, int R, bool TOGETHER>
 cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
                        const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     using T = Traits<KIND>;
-    const long long even = (n + (long long)sh.sms * kRunWarps - 1) / ((long long)sh.sms * kRunWarps);
-    const int run = (int)std::min<long long>(R, (even + 31) / 32 * 32);
+    const long long resident = (long long)sh.sms * run_blocks(Slots<KIND, BB>::KRB, TOGETHER) * 8;
+    const int run = run_length(OP, n, resident, R, (long long)v.nb * BB >= kBeyondReach);
     const long long per_block = (long long)(sh.block / 32) * run;
     const unsigned grid = (unsigned)((n + per_block - 1) / per_block);
     const size_t smem = sizeof(WarpRun<KIND, OP, R>) * (sh.block / 32);

@@ -209,14 +209,16 @@ cudaError_t table_malloc(void **mem, long long bytes, int dev) {
 //   maps   lookups  x = 0.5: present 1.07-1.3, absent 0.73-1.0; 1: 1.25-1.5 and
 //                   0.87-1.4; 2: 1.5-1.7 and 1.1-1.2
 //   sets   lookups  x = 1: 0.9-1.04 and 0.98-2.0; 4: 1.2 and 1.28
-//   inserts         x = 0.25: 0.9-1.3; 0.5: 0.97-1.35; 1: 1.16-1.8; 2: 1.5-1.8
+//   inserts         x = 0.25: 1 GiB 0.9-1.1, 4 GiB 1.08-1.3; 0.5: 0.97-1.35;
+//                   1: 1.16-1.8; 2: 1.5-1.8
 //   erases          x = 0.5: 0.93-1.2; 1: 1.15-1.6
 //   512 MB tables   about twice the x for the same gain; 256 MB: never.
 bool bulk_pays(const hc_table *t, int op, long long n) {
     const long long bytes = (long long)t->view.nb * t->bucket_bytes;
     if (n < (1ll << 21) || bytes < (512ll << 20)) return false;
     const double x = (double)n * 128.0 / (double)bytes;
-    const double large = op == hc::OP_INSERT ? 0.5 : op == hc::OP_ERASE ? 1.0 : is_map(t->kind) ? 1.25 : 1.5;
+    const double large = op == hc::OP_INSERT ? (bytes < (2ll << 30) ? 0.5 : 0.25)
+                         : op == hc::OP_ERASE ? 1.0 : is_map(t->kind) ? 1.25 : 1.5;
     return x >= (bytes < (768ll << 20) ? 2.0 * large + 1.0 : large);
 }
 

@@ -47,6 +47,15 @@ static_assert(sizeof(Traits<KIND_MAP_I64_I32>::Val) <= sizeof(Traits<KIND_MAP_I6
                   sizeof(Traits<KIND_MAP_U64_U64>::Val) <= sizeof(Traits<KIND_MAP_U64_U64>::Key),
               "a lookup's values go over the keys in the scratch");
 
+// The table part of a key: any function of its first bucket that grows with it
+// and has `parts` values.  With the mixing hash the bucket is the upper part of
+// hash * nb, so the hash's upper word serves as well as the bucket.
+__device__ __forceinline__ unsigned part_of(const View &v, unsigned long long key, int parts,
+                                            unsigned long long part_mul) {
+    if (v.hash_mode == HASH_MIX64) return __umulhi((unsigned)(fmix64(key ^ v.seed) >> 32), (unsigned)parts);
+    return (unsigned)__umul64hi(first_bucket(v, key), part_mul);
+}
+
 // The E consecutive elements p[i ..) of an array of m (those inside it), by one
 // load where the array is aligned for it.
 template <class T, int E, class Load, class Load1>
@@ -61,10 +70,11 @@ __device__ __forceinline__ void bulk_load(T (&to)[E], const T *p, int i, int m, 
 
 // Latency of its phases (load, count, scan, place, store) is what bounds the
 // splitting block; reading the keys twice (the second time from L2) instead of
-// keeping them in registers lets three blocks share an SM: 0.097 -> 0.079 ms
-// for 2^24 keys.
+// keeping them in registers lets three or four blocks share an SM (2^24 keys:
+// 0.097 -> 0.079 ms), and the part comes from the hash's upper word (2^26 keys:
+// 0.295 -> 0.264 ms with the fourth block, 18 bytes a key at 4.6 TB/s).
 template <int KIND, bool VALS>
-__global__ void __launch_bounds__(kBulkThreads, 3)
+__global__ void __launch_bounds__(kBulkThreads, VALS ? 3 : 4)
 k_bulk_split(View v, const typename Traits<KIND>::Key *keys, const typename Traits<KIND>::Val *vals, long long n,
              int parts, unsigned long long part_mul, BulkScratch sc) {
     using T = Traits<KIND>;
@@ -99,7 +109,7 @@ k_bulk_split(View v, const typename Traits<KIND>::Key *keys, const typename Trai
 #pragma unroll
         for (int e = 0; e < E; ++e)
             if (i + e < m) {
-                const unsigned p = (unsigned)__umul64hi(first_bucket(v, (unsigned long long)k[e]), part_mul);
+                const unsigned p = part_of(v, (unsigned long long)k[e], parts, part_mul);
                 at[j][e] = p << 16 | atomicAdd(&bins[p], 1u);
             }
     }

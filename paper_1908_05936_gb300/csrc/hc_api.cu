@@ -285,6 +285,39 @@ __global__ void k_rehash_finish(hc::Header *old_h, hc::Header *new_h) {
 
 __global__ void k_clear_err(hc::Header *h) { h->err = 0u; }
 
+// Rehashes t into the uninitialised array behind nv region by region
+// (k_rehash_regions) if the tables are of a size for it and the list of keys
+// left over can be had; *done says whether nv holds every key.
+cudaError_t rehash_by_regions(hc_table *t, const hc::View &nv, cudaStream_t s, bool *done) {
+    *done = false;
+    const unsigned long long bytes = nv.nb * (unsigned long long)t->bucket_bytes;
+    // 16 MB: a few regions per SM; an old array much larger than the new one has
+    // too few blocks to walk it
+    if (nv.hash_mode != hc::HASH_MIX64 || bytes < (16ull << 20) || t->view.nb > 8 * nv.nb) return cudaSuccess;
+    cudaMemPool_t pool = pool_of(t->device);
+    const unsigned long long cap = (unsigned long long)t->phys / 16 + 4096;
+    unsigned long long *list = nullptr;                       // the count, then (256 bytes on) the positions
+    if (!pool || cudaMallocFromPoolAsync(reinterpret_cast<void **>(&list), 256 + cap * 8, pool, s) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return cudaSuccess;
+    }
+    const int sms = sm_count_of(t->device);
+    cudaError_t e;
+    switch (t->kind) {
+        case HC_SET_U32: e = hc::set_u32_rehash_regions(t->view, nv, t->bucket_bytes, list, list + 32, cap, sms, s); break;
+        case HC_SET_U64: e = hc::set_u64_rehash_regions(t->view, nv, t->bucket_bytes, list, list + 32, cap, sms, s); break;
+        case HC_MAP_I64_I32: e = hc::map_i64_i32_rehash_regions(t->view, nv, t->bucket_bytes, list, list + 32, cap, sms, s); break;
+        default: e = hc::map_u64_u64_rehash_regions(t->view, nv, t->bucket_bytes, list, list + 32, cap, sms, s); break;
+    }
+    unsigned long long listed = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&listed, list, sizeof listed, cudaMemcpyDeviceToHost, s);
+    const cudaError_t f = cudaFreeAsync(list, s);
+    if (e == cudaSuccess) e = f;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) *done = listed <= cap;
+    return e;
+}
+
 hc_rc read_header(hc_table *t, hc::Header *out, cudaStream_t s) {
     HC_CUDA(cudaMemcpyAsync(out, t->d_mem, sizeof(hc::Header), cudaMemcpyDeviceToHost, s), "reading the table header");
     HC_CUDA(cudaStreamSynchronize(s), "synchronising the stream");
@@ -644,14 +677,18 @@ hc_rc hc_rehash(hc_table *t, int64_t new_slots, void *stream) {
         return fail(HC_ERR_OOM, "cudaMalloc of %lld bytes failed: %s", (long long)g.bytes, cudaGetErrorString(e));
     }
     hc::View nv = make_view(mem, g, t->view.seed, t->view.hash_mode);
-    e = dispatch_clear(t, nv, g.phys, new_slots, s);
-    const int sms = sm_count_of(t->device);
-    if (e == cudaSuccess) {
-        switch (t->kind) {
-            case HC_SET_U32: e = hc::set_u32_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
-            case HC_SET_U64: e = hc::set_u64_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
-            case HC_MAP_I64_I32: e = hc::map_i64_i32_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
-            default: e = hc::map_u64_u64_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
+    bool done = false;
+    e = rehash_by_regions(t, nv, s, &done);
+    if (e == cudaSuccess && !done) {
+        e = dispatch_clear(t, nv, g.phys, new_slots, s);
+        const int sms = sm_count_of(t->device);
+        if (e == cudaSuccess) {
+            switch (t->kind) {
+                case HC_SET_U32: e = hc::set_u32_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
+                case HC_SET_U64: e = hc::set_u64_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
+                case HC_MAP_I64_I32: e = hc::map_i64_i32_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
+                default: e = hc::map_u64_u64_rehash(t->view, t->phys, nv, t->bucket_bytes, sms, s); break;
+            }
         }
     }
     if (e == cudaSuccess) {

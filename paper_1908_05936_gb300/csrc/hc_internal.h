@@ -31,6 +31,8 @@ struct LaunchShape {
                             uint8_t *out, void *vals_out, int parts, void *scratch, cudaStream_t s);                \
     cudaError_t NAME##_clear(const View &v, unsigned long long phys, unsigned long long cap, int bb, int sms,       \
                              cudaStream_t s);                                                                       \
+    cudaError_t NAME##_rehash_regions(const View &ov, const View &nv, int bb, unsigned long long *count,            \
+                                      unsigned long long *pos, unsigned long long cap, int sms, cudaStream_t s);    \
     cudaError_t NAME##_rehash(const View &ov, unsigned long long ophys, const View &nv, int bb, int sms,            \
                               cudaStream_t s);
 

@@ -105,7 +105,8 @@ __global__ void k_pad_tombstones(View v, unsigned long long first, unsigned long
 // key-dependent slots (View::rotate).  A thread per old slot that looked for an
 // EMPTY slot word by word took 1.69 ms for 2^26 slots of 64-byte buckets at load
 // factor 0.6; the runs take 1.2 ms, bound by instructions (24 warp instructions
-// a key, issue 61 %; DRAM 30 %).
+// a key, issue 61 %; DRAM 30 %).  For small tables and the spatial hashes, whose
+// homes are scattered (next section for the others).
 
 template <int KIND, int BB>
 struct OldSlots {
@@ -145,6 +146,172 @@ k_rehash(View old_v, unsigned long long old_phys, View new_v) {
     insert_run<KIND, BB, false>(new_v, src, (int)(old_phys - first < R ? old_phys - first : R), w.stack, w.st, cnts);
     const unsigned long long busy = (old_phys + R - 1) / R - w0;       // warps of this block with slots
     sum.flush(new_v, cnts, busy < 8 ? (int)busy : 8);
+}
+
+// With the mixing hash a key's new home is at the same share of the new array
+// as its old one of the old array, so the rehash of a large table builds the new
+// array region by region: a block holds kRegionBytes of it in shared memory,
+// walks the same share of the old array, puts each key into its new home or the
+// next bucket of the region with room (a counter per bucket hands out slots),
+// and writes the region out whole, EMPTY slots included.  Keys whose home is
+// elsewhere (their old probe crossed a boundary) or whose probe leaves the
+// region go to a list that is inserted when every region is there; until then no
+// key of the list is looked for, and a bucket that a placed key has passed is
+// full for good.  Every line is read or written once, in order: 2^26 slots of
+// 64-byte buckets at load factor 0.6, 1.37 ms (fill and runs) -> 0.54 ms, 2 GiB
+// at 4 TB/s; what bounds it now is the placing of the keys of a bucket one after
+// another.  32 KB: 512 64-byte buckets, about 1 % of the keys cross a boundary,
+// and six blocks share an SM.
+constexpr int kRegionBytes = 32768;
+
+struct RehashRest {
+    unsigned long long *count;       // keys on the list (may exceed cap: then the list is incomplete)
+    unsigned long long *pos;         // their slot positions in the old array
+    unsigned long long cap;
+};
+
+template <int KIND, int BB>
+__global__ void __launch_bounds__(256)
+k_rehash_regions(View old_v, View new_v, unsigned long long regions, RehashRest rest) {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using Val = typename T::Val;
+    using S = Slots<KIND, BB>;
+    constexpr int SPB = S::SPB, M = kRegionBytes / BB;
+    __shared__ __align__(16) unsigned char region[kRegionBytes];
+    constexpr unsigned kListed = 256;                         // keys on a block's part of the list
+    __shared__ unsigned taken[M];
+    __shared__ unsigned long long listed[kListed], list_base;
+    __shared__ unsigned n_listed;
+    __shared__ BlockCounts sum;
+    const int tid = threadIdx.x;
+    const unsigned long long g = blockIdx.x;
+    const unsigned long long n0 = g * new_v.nb / regions, n1 = (g + 1) * new_v.nb / regions;
+    const unsigned long long o0 = g * old_v.nb / regions, o1 = (g + 1) * old_v.nb / regions;
+    const int size = (int)(n1 - n0);                          // buckets of this region, at most M
+    for (int i = tid; i < kRegionBytes / 16; i += 256) reinterpret_cast<uint4 *>(region)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    for (int i = tid; i < M; i += 256) taken[i] = 0u;
+    if (tid == 0) n_listed = 0u;
+    sum.init();
+    // the last bucket's padding: never handed out, tombstones
+    const int last = n1 == new_v.nb ? size - 1 : -1;
+    if (last >= 0)
+        for (int x = new_v.pad_from + tid; x < SPB; x += 256)
+            *reinterpret_cast<Key *>(region + last * BB + x * S::KB) = T::TOMB;
+    Counts cnts;
+    for (unsigned long long ob0 = o0; ob0 < o1; ob0 += 256) {
+        const unsigned long long ob = ob0 + tid;
+        LaneWords<S::KRB> kw;
+        uint32_t live = 0;
+        Val val[T::MAP ? SPB : 1];
+        if (ob < o1) {
+            kw.load(bucket_at<BB>(old_v, ob));
+#pragma unroll
+            for (int x = 0; x < SPB; ++x) {
+                const Key k = slot_key<KIND, S::KRB>(kw, x);
+                live |= (uint32_t)(k != T::EMPTY && k != T::TOMB) << x;
+            }
+            if constexpr (T::MAP) {
+                if (live) {
+                    constexpr int VRB = SPB * (int)sizeof(Val);
+                    const unsigned char *p = bucket_at<BB>(old_v, ob) + S::KRB;
+                    if constexpr (VRB >= 16) {
+#pragma unroll
+                        for (int q = 0; q < VRB / 16; ++q) {
+                            const uint4 u = __ldcs(reinterpret_cast<const uint4 *>(p) + q);
+                            memcpy(&val[q * 16 / (int)sizeof(Val)], &u, 16);
+                        }
+                    } else {
+                        const uint2 u = __ldcs(reinterpret_cast<const uint2 *>(p));
+                        memcpy(&val[0], &u, 8);
+                    }
+                }
+            }
+        }
+        uint32_t over = 0;                                    // slots whose keys go to the list
+#pragma unroll
+        for (int x = 0; x < SPB; ++x) {
+            if (!(live >> x & 1u)) continue;
+            const Key k = slot_key<KIND, S::KRB>(kw, x);
+            const unsigned long long home = first_bucket(new_v, (unsigned long long)k);
+            bool placed = false;
+            if (home >= n0 && home < n1) {
+                for (int b = (int)(home - n0); b < size && !placed; ++b) {
+                    const unsigned room = b == last ? (unsigned)new_v.pad_from : (unsigned)SPB;
+                    if (*(volatile unsigned *)&taken[b] >= room) continue;
+                    const unsigned s = atomicAdd(&taken[b], 1u);
+                    if (s >= room) continue;
+                    *reinterpret_cast<Key *>(region + b * BB + s * S::KB) = k;
+                    if constexpr (T::MAP) {
+                        *reinterpret_cast<Val *>(region + b * BB + S::KRB + s * S::VB) = val[x];
+                        note_claim_key<KIND>(new_v.hdr, k, (long long)((n0 + b) * SPB + s));
+                    }
+                    placed = true;
+                }
+            }
+            cnts.new_slot += placed;
+            over |= (uint32_t)!placed << x;
+        }
+#pragma unroll
+        for (int x = 0; x < SPB; ++x) {
+            if (!(over >> x & 1u)) continue;
+            const unsigned at = atomicAdd(&n_listed, 1u);
+            if (at < kListed) {
+                listed[at] = ob * SPB + x;
+            } else {
+                const unsigned long long to = atomicAdd(rest.count, 1ull);
+                if (to < rest.cap) rest.pos[to] = ob * SPB + x;
+            }
+        }
+    }
+    __syncthreads();
+    const int mine = (int)(n_listed < kListed ? n_listed : kListed);
+    if (tid == 0) list_base = mine ? atomicAdd(rest.count, (unsigned long long)mine) : 0ull;
+    __syncthreads();
+    uint4 *out = reinterpret_cast<uint4 *>(new_v.buckets + n0 * BB);
+    for (int i = tid; i < size * BB / 16; i += 256) out[i] = reinterpret_cast<const uint4 *>(region)[i];
+    __syncthreads();
+    for (int i = tid; i < mine; i += 256)
+        if (list_base + i < rest.cap) rest.pos[list_base + i] = listed[i];
+    sum.flush(new_v, cnts, 8);
+}
+
+template <int KIND, int BB>
+struct ListedSlots {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using Val = typename T::Val;
+    using S = Slots<KIND, BB>;
+    const View &old_v;
+    const unsigned long long *pos;
+    unsigned long long p = 0;
+    __device__ __forceinline__ Key key(int i) {
+        p = pos[i];
+        return *reinterpret_cast<const Key *>(S::key(old_v, p / S::SPB, (int)(p % S::SPB)));
+    }
+    __device__ __forceinline__ bool skip(int) const { return false; }
+    __device__ __forceinline__ Val val(int) const {          // of the key asked for last
+        return *reinterpret_cast<const Val *>(S::val(old_v, p / S::SPB, (int)(p % S::SPB)));
+    }
+};
+
+// The listed keys, in runs that the grid's warps stride over.
+template <int KIND, int BB>
+__global__ void __launch_bounds__(256, run_blocks(Slots<KIND, BB>::KRB, false))
+k_rehash_rest(View old_v, View new_v, RehashRest rest) {
+    constexpr int R = 64;
+    __shared__ WarpRun<KIND, OP_INSERT, R> sh[8];
+    __shared__ BlockCounts sum;
+    sum.init();
+    WarpRun<KIND, OP_INSERT, R> &w = sh[threadIdx.x >> 5];
+    const unsigned long long n = *rest.count < rest.cap ? *rest.count : rest.cap;
+    const unsigned long long stride = (unsigned long long)gridDim.x * 8 * R;
+    Counts cnts;
+    for (unsigned long long first = ((unsigned long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * R; first < n; first += stride) {
+        ListedSlots<KIND, BB> src{old_v, rest.pos + first};
+        insert_run<KIND, BB, false>(new_v, src, (int)(n - first < R ? n - first : R), w.stack, w.st, cnts);
+    }
+    sum.flush(new_v, cnts, 8);
 }
 
 // ------------------------------------------------------------ launchers ---
@@ -396,6 +563,27 @@ cudaError_t launch_clear(const View &v, unsigned long long phys, unsigned long l
 }
 
 template <int KIND>
+cudaError_t launch_rehash_regions(const View &old_v, const View &new_v, int bucket_bytes, unsigned long long *count,
+                                  unsigned long long *pos, unsigned long long cap, int sms, cudaStream_t s) {
+    const RehashRest rest{count, pos, cap};
+    const unsigned long long most = kRegionBytes / bucket_bytes, regions = (new_v.nb + most - 1) / most;
+    cudaError_t e = cudaMemsetAsync(new_v.hdr, 0, sizeof(Header), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof *count, s);
+    if (e != cudaSuccess) return e;
+    const unsigned few = (unsigned)(sms * 4);
+    switch (bucket_bytes) {
+        case 32: k_rehash_regions<KIND, 32><<<(unsigned)regions, 256, 0, s>>>(old_v, new_v, regions, rest);
+                 k_rehash_rest<KIND, 32><<<few, 256, 0, s>>>(old_v, new_v, rest); break;
+        case 64: k_rehash_regions<KIND, 64><<<(unsigned)regions, 256, 0, s>>>(old_v, new_v, regions, rest);
+                 k_rehash_rest<KIND, 64><<<few, 256, 0, s>>>(old_v, new_v, rest); break;
+        case 128: k_rehash_regions<KIND, 128><<<(unsigned)regions, 256, 0, s>>>(old_v, new_v, regions, rest);
+                  k_rehash_rest<KIND, 128><<<few, 256, 0, s>>>(old_v, new_v, rest); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+template <int KIND>
 cudaError_t launch_rehash(const View &old_v, unsigned long long old_phys, const View &new_v, int bucket_bytes,
                           int sm_count, cudaStream_t s) {
     (void)sm_count;
@@ -428,6 +616,10 @@ cudaError_t launch_rehash(const View &old_v, unsigned long long old_phys, const 
     cudaError_t NAME##_clear(const View &v, unsigned long long phys, unsigned long long cap, int bb, int sms,       \
                              cudaStream_t s) {                                                                      \
         return launch_clear<KIND>(v, phys, cap, bb, sms, s);                                                        \
+    }                                                                                                               \
+    cudaError_t NAME##_rehash_regions(const View &ov, const View &nv, int bb, unsigned long long *count,            \
+                                      unsigned long long *pos, unsigned long long cap, int sms, cudaStream_t s) {   \
+        return launch_rehash_regions<KIND>(ov, nv, bb, count, pos, cap, sms, s);                                    \
     }                                                                                                               \
     cudaError_t NAME##_rehash(const View &ov, unsigned long long ophys, const View &nv, int bb, int sms,            \
                               cudaStream_t s) {                                                                     \

@@ -6,15 +6,20 @@
 // the in-kernel functions of include/hc_device.cuh do (whose waiting rule and
 // special keys it shares).
 //
-// The kernel has the shape of the streaming range kernels: a block stages its
-// chunk of operations, keys and values in shared memory with 16-byte loads,
-// every thread keeps S operations in flight and refills a slot from the chunk
-// as soon as its operation finishes, and in each round all the round's
-// compare-and-swaps go out together.  A map insert's claim and its publication
-// happen in the same round, around one fence per thread and round that also
-// orders the round's lookups of found keys before their value reads; no claim
-// is left in progress from one round to the next, so a wait on a claim always
-// ends.  Results leave in coalesced stores, counters with one atomic per warp.
+// The kernel has the shape of the range kernels (warp runs): a warp works
+// through a run of operations, those that stay undecided wait on its stack.  In
+// a step all compare-and-swaps go out together; a map insert's claim and its
+// publication happen in the same step, around one fence that also orders the
+// step's lookups of found keys before their value reads; no claim is left in
+// progress from one step to the next, so a wait on a claim always ends.  Results
+// leave in coalesced stores, counters with one atomic per block.
+//
+// Against a kernel that staged a block's operations and kept two per thread in
+// flight (50 / 30 / 20 inserts, lookups, erases): 2^22 on a 256 MB map 236 -> 216
+// us, on a 256 MB set 149 -> 130, 2^18 on a 16 MB map 50 -> 32, 2^24 on a 4 GiB
+// map 1.08 -> 1.06 ms; what bounds the large ones is a map insert's three
+// scattered requests (claim, value, key) after its read.  Eight blocks per SM (64
+// registers): without the cap 244 us for the first, at ten 1.09 ms for the last.
 #include <algorithm>
 #include <cstdint>
 
@@ -27,9 +32,8 @@ namespace hc {
 
 namespace {
 
-constexpr int kMixedBlock = 64;   // threads per block
-constexpr int kMixedKPT = 8;      // operations per thread per chunk
-constexpr int kMixedS = 2;        // operations in flight per thread
+constexpr int kMixedBlock = 128;  // threads per block
+constexpr int kMixedRun = 128;    // operations per run at most
 
 enum : uint8_t { MOP_INSERT = 0, MOP_FIND = 1, MOP_ERASE = 2 };
 
@@ -53,233 +57,223 @@ __device__ __noinline__ void special_op(const View &v, uint8_t op, typename Trai
     }
 }
 
-template <int KIND, int BB, int KPT, int S>
-__global__ void __launch_bounds__(256)
-k_mixed_stream(View v, const uint8_t *ops, const typename Traits<KIND>::Key *keys,
-               const typename Traits<KIND>::Val *vals, long long n, uint8_t *status,
-               typename Traits<KIND>::Val *vals_out) {
+// The operations in flight of a warp: key, bucket << 16 | kind << 14 | position
+// in the run, an insert's value.
+template <int KIND>
+struct MixedRun {
+    using T = Traits<KIND>;
+    unsigned long long at[kStack];
+    typename T::Key key[kStack];
+    typename T::Val val[T::MAP ? kStack : 1];
+    typename T::Val vals[T::MAP ? kMixedRun : 1];            // found values out
+    uint8_t st[kMixedRun];
+};
+
+template <int KIND, int BB>
+__global__ void __launch_bounds__(kMixedBlock, 8)
+k_mixed_run(View v, const uint8_t *ops, const typename Traits<KIND>::Key *keys, const typename Traits<KIND>::Val *vals,
+            long long n, int run, uint8_t *status, typename Traits<KIND>::Val *vals_out) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
     using Sl = Slots<KIND, BB>;
-    constexpr int LB = Sl::KRB;              // one thread reads the whole key region
-    constexpr int SPB = Sl::SPB;
-    constexpr int VB = T::MAP ? (int)sizeof(Val) : 0;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int nt = blockDim.x;
-    const int chunk = nt * KPT;
-    const long long c0 = (long long)blockIdx.x * chunk;
-    const int m = (int)(n - c0 < chunk ? n - c0 : chunk);
-    debug_range(v, c0, m, n);
-    Key *sk = reinterpret_cast<Key *>(smem);
-    Val *sv = reinterpret_cast<Val *>(smem + (size_t)chunk * sizeof(Key));   // values in, found values out
-    uint8_t *so = smem + (size_t)chunk * (sizeof(Key) + VB);                  // operation kinds
-    uint8_t *ss = so + chunk;                                                 // results
+    constexpr int SPB = Sl::SPB, WARPS = kMixedBlock / 32;
+    __shared__ MixedRun<KIND> sh[WARPS];
+    __shared__ BlockCounts sum;
+    sum.init();
+    MixedRun<KIND> &w = sh[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const long long w0 = (long long)blockIdx.x * WARPS;
+    const long long c0 = (w0 + (threadIdx.x >> 5)) * run;
+    if (c0 >= n) return;
+    const int cnt = (int)(n - c0 < run ? n - c0 : run);
+    debug_range(v, c0, cnt, n);
+    keys += c0;
+    ops += c0;
+    if constexpr (T::MAP) vals += c0;
 
-    Stage<Key, KPT> gk;
-    Stage<Val, KPT> gv;
-    Stage<uint8_t, KPT> go;
-    gk.load(keys + c0, m);
-    if constexpr (T::MAP) gv.load(vals + c0, m);
-    go.load(ops + c0, m);
-    gk.store(sk, m);
-    if constexpr (T::MAP) gv.store(sv, m);
-    go.store(so, m, [](uint8_t o) { return o == MOP_INSERT ? (uint8_t)MOP_INSERT : (o == MOP_FIND ? (uint8_t)MOP_FIND : (uint8_t)MOP_ERASE); });
-    __syncthreads();
-
-    Counts cnt;
-    int idx[S];
-    Key key[S];
-    uint8_t op[S];
-    unsigned long long b[S];
-    uint32_t probes[S], retries[S];
-    int qs[S];
-    int next = 0;
-    uint32_t active = 0;
-    auto take = [&](int s) {
-        while (next < KPT) {
-            const int i = threadIdx.x + (next++) * nt;
-            if (i >= m) { next = KPT; break; }
-            const Key k = sk[i];
-            const uint8_t o = so[i];
-            bool special = side_index<KIND>(k) >= 0;
-            if constexpr (T::MAP) special = special || k == T::CLAIM;
-            if (special) {
-                Val dummy = Val();
-                special_op<KIND, BB>(v, o, k, T::MAP ? &sv[i] : &dummy, &ss[i]);
-                continue;
-            }
-            idx[s] = i;
-            key[s] = k;
-            op[s] = o;
-            b[s] = first_bucket(v, (unsigned long long)k);
-            probes[s] = 0;
-            retries[s] = 0;
-            active |= 1u << s;
-            return;
-        }
+    Counts cnts;
+    int next = 0, top = 0;
+    Key ahead = Key();
+    Val ahead_val = Val();
+    uint8_t ahead_op = 0;
+    auto fetch = [&](int i) {
+        if (i >= cnt) return;
+        ahead = ld_stream(keys + i);
+        if constexpr (T::MAP) ahead_val = ld_stream(vals + i);
+        ahead_op = ld_stream(ops + i);
     };
-    // an operation is over: its result byte is written; a map's value slot
-    // keeps a found value (finds) or becomes 0 (inserts, erases)
-    auto done = [&](int s, uint8_t st, uint32_t &finished) {
-        ss[idx[s]] = st;
-        if constexpr (T::MAP) {
-            if (op[s] != MOP_FIND || st == 0) sv[idx[s]] = Val();
-        }
-        finished |= 1u << s;
-    };
-#pragma unroll
-    for (int s = 0; s < S; ++s) take(s);
-    while (active) {
-        LaneWords<LB> lw[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-            if (active >> s & 1u) lw[s].load(bucket_at<BB>(v, b[s]));
-        uint32_t finished = 0, swapping = 0, reading = 0;
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(active >> s & 1u)) continue;
-            uint32_t lm = 0, le = 0, lc = 0;
-#pragma unroll
-            for (int q = 0; q < SPB; ++q) {
-                const Key ks = slot_key<KIND, LB>(lw[s], q);
-                lm |= (uint32_t)(ks == key[s]) << q;
-                le |= (uint32_t)(ks == T::EMPTY) << q;
-                if constexpr (T::MAP) lc |= (uint32_t)(ks == T::CLAIM) << q;
+    fetch(lane);
+    unsigned long long reach = 0;
+    for (;; ++reach) {
+        Key key;
+        Val val = Val();
+        uint8_t op;
+        unsigned long long b = 0;
+        int idx;
+        bool act;
+        if (top < 32 && next < cnt) {
+            key = ahead;
+            val = ahead_val;
+            op = ahead_op == MOP_INSERT ? MOP_INSERT : ahead_op == MOP_FIND ? MOP_FIND : MOP_ERASE;
+            idx = next + lane;
+            act = idx < cnt;
+            next += 32;
+            fetch(next + lane);
+            bool special = side_index<KIND>(key) >= 0;
+            if constexpr (T::MAP) special = special || key == T::CLAIM;
+            if (act && special) {
+                Val out = val;
+                special_op<KIND, BB>(v, op, key, &out, &w.st[idx]);
+                if constexpr (T::MAP) w.vals[idx] = out;
+                act = false;
             }
-            if (op[s] == MOP_FIND) {
-                if (lm) {
-                    if constexpr (T::MAP) {          // the value is read after this round's fence
-                        qs[s] = __ffs(lm) - 1;
-                        reading |= 1u << s;
-                    } else {
-                        done(s, 1, finished);
-                    }
-                } else if (le || ++probes[s] >= v.nb) {
-                    done(s, 0, finished);
-                } else {
-                    b[s] = next_bucket(v, b[s]);
-                }
-            } else if (op[s] == MOP_ERASE) {
-                if (lm) {
-                    qs[s] = __ffs(lm) - 1;
-                    swapping |= 1u << s;
-                } else if (le || ++probes[s] >= v.nb) {
-                    done(s, ST_NOT_FOUND, finished);
-                } else {
-                    b[s] = next_bucket(v, b[s]);
-                }
-            } else {
-                if (lm) {                            // stored (and, for maps, published with its value)
-                    done(s, ST_EXISTS, finished);
-                    continue;
-                }
-                const int rot = slot_rotation<SPB>((unsigned long long)key[s]);
+            b = first_bucket(v, (unsigned long long)key);
+        } else if (top > 0) {
+            const int take = top < 32 ? top : 32;
+            top -= take;
+            act = lane < take;
+            const int p = top + (act ? lane : 0);
+            const unsigned long long e = w.at[p];
+            key = w.key[p];
+            if constexpr (T::MAP) val = w.val[p];
+            idx = (int)(e & 0x3fffu);
+            op = (uint8_t)(e >> 14 & 3u);
+            b = e >> 16;
+        } else {
+            break;
+        }
+        __syncwarp();                        // entries are read before this step's survivors overwrite them
+        const Seen seen = see_bucket<KIND, BB, false, true>(v, act, b, key);
+        // an operation is over with result st; a map's value is 0 but for a found key
+        bool left = act;
+        auto done = [&](uint32_t st) {
+            w.st[idx] = (uint8_t)st;
+            if constexpr (T::MAP) w.vals[idx] = Val();
+            left = false;
+        };
+        int q = -1;                          // the slot of this step's swap, or of a found key's value
+        bool swap = false;
+        if (act) {
+            const uint32_t le = seen.empty;
+            bool full = false;
+            if (op == MOP_INSERT) {
+                const int rot = slot_rotation<SPB>((unsigned long long)key);
                 bool wait = false;
-                if constexpr (T::MAP) {              // the stored CLAIM-pattern key, or claims in progress
-                    if (lc) wait = hcd::detail::must_wait<SPB>(v, b[s], lc, le, rot);
-                }
-                if (wait) {                          // read the bucket again next round
-                    if (++retries[s] > kMaxRestarts) {
-                        atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
-                        cnt.over = 1;
-                        done(s, ST_OVERFLOW, finished);
+                if (seen.hit) {              // stored (and, for maps, published with its value)
+                    done(ST_EXISTS);
+                } else {
+                    if constexpr (T::MAP) {  // the stored CLAIM-pattern key, or claims in progress
+                        if (seen.tomb) wait = hcd::detail::must_wait<SPB>(v, b, seen.tomb, le, rot);
                     }
-                } else if (!le) {
-                    if (++probes[s] >= v.nb) {
-                        cnt.over = 1;
-                        done(s, ST_OVERFLOW, finished);
+                    if (wait) {              // the bucket is read again
+                        full = false;
+                    } else if (le) {
+                        q = hcd::detail::first_from<SPB>(le, rot);
+                        swap = true;
                     } else {
-                        b[s] = next_bucket(v, b[s]);
+                        full = true;
                     }
-                } else {
-                    qs[s] = hcd::detail::first_from<SPB>(le, rot);
-                    swapping |= 1u << s;
                 }
+            } else if (seen.hit) {
+                q = __ffs(seen.hit) - 1;
+                swap = op == MOP_ERASE;
+                if constexpr (!T::MAP) {
+                    if (!swap) done(1u);
+                }
+            } else if (le) {
+                done(op == MOP_FIND ? 0u : (uint32_t)ST_NOT_FOUND);
+            } else {
+                full = true;
+            }
+            if (full) {
+                b = next_bucket(v, b);
+                if (came_round(v, (unsigned long long)key, b, reach)) {
+                    if (op == MOP_INSERT) cnts.over = 1;
+                    done(op == MOP_INSERT ? (uint32_t)ST_OVERFLOW : op == MOP_FIND ? 0u : (uint32_t)ST_NOT_FOUND);
+                }
+            } else if (left && !swap && q < 0 && reach >= v.nb + 32ull * kMaxRestarts) {
+                atomicOr(&v.hdr->err, ERR_PROBE_BOUND);      // a claim that never resolves
+                cnts.over = 1;
+                done(ST_OVERFLOW);
             }
         }
-        Key old[S];
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(swapping >> s & 1u)) continue;
-            unsigned char *slot = Sl::key(v, b[s], qs[s]);
-            if (op[s] == MOP_ERASE) old[s] = cas_key<KIND>(slot, key[s], T::TOMB);
-            else old[s] = cas_key<KIND>(slot, T::EMPTY, T::MAP ? T::CLAIM : key[s]);
-        }
-        uint32_t publishing = 0;
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (!(swapping >> s & 1u)) continue;
-            if (op[s] == MOP_ERASE) {
+        bool publish = false;
+        if (swap) {
+            unsigned char *slot = Sl::key(v, b, q);
+            if (op == MOP_ERASE) {
                 // a failed swap means a concurrent erase of the same key won
-                const bool won = old[s] == key[s];
-                cnt.del += won ? 1u : 0u;
-                done(s, won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND, finished);
-            } else if (old[s] == T::EMPTY) {
-                if constexpr (T::MAP) {
-                    store_val<KIND, BB>(v, b[s], qs[s], (unsigned long long)sv[idx[s]]);
-                    publishing |= 1u << s;
-                } else {
-                    ++cnt.ins;
-                    ++cnt.new_slot;
-                    done(s, ST_INSERTED, finished);
+                const bool won = cas_key<KIND>(slot, key, T::TOMB) == key;
+                cnts.del += won ? 1u : 0u;
+                done(won ? (uint32_t)ST_ERASED : (uint32_t)ST_NOT_FOUND);
+            } else {
+                const Key old = cas_key<KIND>(slot, T::EMPTY, T::MAP ? T::CLAIM : key);
+                if (old == T::EMPTY) {
+                    ++cnts.ins;
+                    ++cnts.new_slot;
+                    if constexpr (T::MAP) {
+                        store_val<KIND, BB>(v, b, q, (unsigned long long)val);
+                        publish = true;
+                    } else {
+                        done(ST_INSERTED);
+                    }
+                } else if (!T::MAP && old == key) {
+                    done(ST_EXISTS);         // an equal key won the slot
+                } else if (reach >= v.nb + 32ull * kMaxRestarts) {
+                    atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
+                    cnts.over = 1;
+                    done(ST_OVERFLOW);
                 }
-            } else if (!T::MAP && old[s] == key[s]) {
-                done(s, ST_EXISTS, finished);        // an equal key won the slot
-            } else if (++retries[s] > kMaxRestarts) {
-                atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
-                cnt.over = 1;
-                done(s, ST_OVERFLOW, finished);
+                // otherwise another key took the slot: the same bucket is read again
             }
-            // otherwise another key took the slot: the same bucket is read again
         }
         if constexpr (T::MAP) {
-            if (publishing | reading) {
+            const bool reading = act && left && op == MOP_FIND && q >= 0;
+            if (publish || reading) {
                 // the claimed slots' values before their keys; the found keys'
                 // loads before their values' loads
                 __threadfence();
-#pragma unroll
-                for (int s = 0; s < S; ++s) {
-                    if (publishing >> s & 1u) {
-                        hcd::detail::store_key<KIND>(Sl::key(v, b[s], qs[s]), key[s]);
-                        ++cnt.ins;
-                        ++cnt.new_slot;
-                        done(s, ST_INSERTED, finished);
-                    } else if (reading >> s & 1u) {
-                        sv[idx[s]] = (Val)load_val<KIND, BB>(v, b[s], qs[s]);
-                        done(s, 1, finished);
-                    }
+                if (publish) {
+                    hcd::detail::store_key<KIND>(Sl::key(v, b, q), key);
+                    done(ST_INSERTED);
+                } else {
+                    w.vals[idx] = (Val)load_val<KIND, BB>(v, b, q);
+                    w.st[idx] = 1;
+                    left = false;
                 }
             }
         }
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            if (finished >> s & 1u) {
-                active &= ~(1u << s);
-                take(s);
-            }
+        const unsigned mask = __ballot_sync(0xffffffffu, left);
+        if (left) {
+            const int p = top + __popc(mask & lanes_below());
+            w.at[p] = b << 16 | (unsigned)op << 14 | (unsigned)idx;
+            w.key[p] = key;
+            if constexpr (T::MAP) w.val[p] = val;
         }
+        top += __popc(mask);
+        __syncwarp();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += nt) {
-        if (status) st_stream(status + c0 + i, ss[i]);
+    __syncwarp();
+    for (int i = lane; i < cnt; i += 32) {
+        if (status) st_stream(status + c0 + i, w.st[i]);
         if constexpr (T::MAP) {
-            if (vals_out) st_stream(vals_out + c0 + i, sv[i]);
+            if (vals_out) st_stream(vals_out + c0 + i, w.vals[i]);
         }
     }
-    flush_counts(v, cnt);
+    const long long busy = (n + run - 1) / run - w0;         // warps of this block with operations
+    sum.flush(v, cnts, (int)(busy < WARPS ? busy : WARPS));
 }
 
 template <int KIND, int BB>
 cudaError_t launch_bb(const View &v, const uint8_t *ops, const void *keys, const void *vals, long long n,
                       uint8_t *status, void *vals_out, cudaStream_t s) {
     using T = Traits<KIND>;
-    constexpr int chunk = kMixedBlock * kMixedKPT;
-    const size_t smem = (size_t)chunk * (sizeof(typename T::Key) + (T::MAP ? sizeof(typename T::Val) : 0) + 2);
-    const unsigned grid = (unsigned)((n + chunk - 1) / chunk);
-    k_mixed_stream<KIND, BB, kMixedKPT, kMixedS><<<grid, kMixedBlock, smem, s>>>(
-        v, ops, (const typename T::Key *)keys, (const typename T::Val *)vals, n, status,
-        (typename T::Val *)vals_out);
+    // at least 32 warps on each of 128 SMs before runs grow
+    const int run = (int)std::min<long long>(kMixedRun, (n + 4096 * 32 - 1) / (4096 * 32) * 32);
+    const long long per_block = (long long)(kMixedBlock / 32) * run;
+    const unsigned grid = (unsigned)((n + per_block - 1) / per_block);
+    k_mixed_run<KIND, BB><<<grid, kMixedBlock, 0, s>>>(v, ops, (const typename T::Key *)keys, (const typename T::Val *)vals,
+                                                       n, run, status, (typename T::Val *)vals_out);
     return cudaGetLastError();
 }
 

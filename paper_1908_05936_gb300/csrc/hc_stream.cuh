@@ -181,7 +181,8 @@ struct Drain {
     }
 };
 
-// What a key finds in a bucket, one bit per slot.
+// What a key finds in a bucket, one bit per slot (free-running batches look for
+// claims in progress in place of tombstones).
 struct Seen {
     uint32_t hit, empty, tomb;
 };
@@ -198,13 +199,14 @@ struct Seen {
 // 13.7 -> 23.8, 64 MB 34.8 -> 28.9; map<i64,i32>, 128-byte buckets (64 of keys):
 // 512 MB 20.8 -> 28.1, 256 MB (2^20, load factor 0.7) 29.9 -> 30.1, its inserts
 // 15.2 -> 13.1.
-template <int KIND, int BB, bool TOGETHER>
+template <int KIND, int BB, bool TOGETHER, bool CLAIMS = false>
 __device__ __forceinline__ Seen see_bucket(const View &v, bool act, unsigned long long b,
                                            typename Traits<KIND>::Key key) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Sl = Slots<KIND, BB>;
     constexpr int SPB = Sl::SPB;
+    constexpr Key MARK = CLAIMS ? T::CLAIM : T::TOMB;
     if constexpr (!TOGETHER || Sl::KRB <= 32) {
         Seen m{0u, 0u, 0u};
         if (act) {
@@ -215,7 +217,7 @@ __device__ __forceinline__ Seen see_bucket(const View &v, bool act, unsigned lon
                 const Key ks = slot_key<KIND, Sl::KRB>(lw, x);
                 m.hit |= (uint32_t)(ks == key) << x;
                 m.empty |= (uint32_t)(ks == T::EMPTY) << x;
-                m.tomb |= (uint32_t)(ks == T::TOMB) << x;
+                m.tomb |= (uint32_t)(ks == MARK) << x;
             }
         }
         return m;
@@ -240,7 +242,7 @@ __device__ __forceinline__ Seen see_bucket(const View &v, bool act, unsigned lon
                     const Key ks = slot_key<KIND, 32>(lw[r], x);
                     m.hit |= (uint32_t)(ks == rk) << x;
                     m.empty |= (uint32_t)(ks == T::EMPTY) << x;
-                    m.tomb |= (uint32_t)(ks == T::TOMB) << x;
+                    m.tomb |= (uint32_t)(ks == MARK) << x;
                 }
             }
             if constexpr (SPB <= 8) {

@@ -246,9 +246,13 @@ cudaError_t try_bulk(hc_table *t, int op, const hc::View &v, const void *keys, c
     }
     cudaMemPool_t pool = pool_of(t->device);
     if (!pool) return cudaSuccess;
-    // parts of about 32 MB: two of them and the keys in flight stay in L2
+    // Parts of 16 to 32 MB, 64 or a multiple of it: a chunk's runs then have 64
+    // keys or fewer, and whole runs fill a probing warp's 256 places to three
+    // quarters or more (32 parts: one run of 128; 1 GiB tables, 32 -> 64 parts:
+    // set inserts 27.3 -> 30.1 G/s, map inserts 17.9 -> 18.5, lookups the same;
+    // 128 parts of 8 MB: map lookups 42.0 -> 40.7).
     const long long bytes = (long long)v.nb * t->bucket_bytes;
-    const int parts = (int)std::min<long long>(hc::kBulkParts, (bytes + (32ll << 20) - 1) / (32ll << 20));
+    const int parts = (int)std::min<long long>(hc::kBulkParts, (bytes + (2ll << 30) - 1) / (2ll << 30) * 64);
     void *scratch = nullptr;
     const long long need = hc::bulk_scratch(nullptr, nullptr, std::min(n, hc::kBulkPiece), parts, key_bytes(t->kind),
                                             val_bytes(t->kind), op);

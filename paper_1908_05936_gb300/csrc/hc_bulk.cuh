@@ -28,7 +28,9 @@
 // 0.55 -> 0.8 12.8 -> 22.3, erases 22.2 -> 34.9; 2^26 lookups, half present, at
 // 0.8: 3.56 -> 1.99 ms; 30 M set lookups on 10^8 slots 0.84 -> 0.62 ms; the
 // 2^28-slot step 25.3 -> 16.1 ms.
-// Parts of 32 MB: 16 or 64 MB are within 3 %.  256 keys a warp: with 512 or more
+// Parts of 32 MB: 16 or 64 MB are within 3 % (4 GiB).  Bringing the next parts
+// into L2 ahead of the probes by bulk prefetches loses at every distance from 8
+// to 96 MB (lookups 43 -> 32-36 G/s).  256 keys a warp: with 512 or more
 // the parts in flight no longer fit L2 (erases 33 -> 28 G/s), with 128 the ends
 // of the runs cost more.
 #pragma once

@@ -203,6 +203,7 @@ k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
+    constexpr bool WHOLE = T::MAP && OP == OP_FIND && BB == 32;    // (2^26 present ones, 4 GiB: 37.4 -> 40.8 G/s)
     __shared__ WarpRun<KIND, OP, R> sh[NT / 32];
     __shared__ unsigned s_start[NT / 32][32], s_upto[NT / 32][32];
     __shared__ BlockCounts sum;
@@ -238,7 +239,7 @@ k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs
         __syncwarp();
         RunsSrc<KIND> src{reinterpret_cast<const Key *>(sc.keys), reinterpret_cast<const Val *>(sc.vals), start, upto};
         if constexpr (OP == OP_INSERT) insert_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
-        else if constexpr (OP == OP_FIND) find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals);
+        else if constexpr (OP == OP_FIND) find_run<KIND, BB, WHOLE>(v, src, m, w.stack, w.st, w.vals);
         else erase_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
         for (int i = lane; i < m; i += 32) {
             const unsigned to = src.place(i);

@@ -368,6 +368,8 @@ inline int run_length(int op, long long n, long long resident, int most, bool be
 // Tables from which lanes read wide buckets together (see_bucket; between 256
 // MB, where it costs 0-17 %, and 512 MB, where it gains 5-50 %).
 constexpr long long kTogetherBytes = kBeyondReach;
+// Maps with 32-byte buckets of which lookups read whole buckets (see_whole_bucket).
+constexpr long long kWholeBytes = 256ll << 20;
 
 template <int KIND, int BB, int OP, int R, bool TOGETHER>
 cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
@@ -389,6 +391,10 @@ cudaError_t launch_run(const View &v, const void *keys, const void *vals, long l
                        const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     if constexpr (Slots<KIND, BB>::KRB > 32) {
         if ((long long)v.nb * BB >= kTogetherBytes)
+            return launch_run_as<KIND, BB, OP, R, true>(v, keys, vals, n, out, vals_out, sh, skip, s);
+    }
+    if constexpr (OP == OP_FIND && Traits<KIND>::MAP && BB == 32) {
+        if ((long long)v.nb * BB >= kWholeBytes)
             return launch_run_as<KIND, BB, OP, R, true>(v, keys, vals, n, out, vals_out, sh, skip, s);
     }
     return launch_run_as<KIND, BB, OP, R, false>(v, keys, vals, n, out, vals_out, sh, skip, s);

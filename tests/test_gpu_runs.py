@@ -82,3 +82,34 @@ def test_batches_at_the_edges_of_steps_and_runs(kind, bb, kpt):
         p.check()
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("kind", (O.MAP_I64_I32, O.MAP_U64_U64))
+@pytest.mark.parametrize("slots", ((1 << 24) - 1, (1 << 24) + 1))
+def test_whole_bucket_lookups(kind, slots):
+    """Maps with 32-byte buckets just below and from 256 MB on, where a lookup
+    reads keys and values together, against the lookup of one key per lane
+    group: hits in either slot, misses, tombstones and reserved keys."""
+    import torch
+
+    from paper_1908_05936_gb300.table import VAL_BYTES, Table
+    width = torch.int64 if VAL_BYTES[kind] == 8 else torch.int32
+    g = torch.Generator(device="cuda").manual_seed(kind)
+    keys = torch.randint(-(1 << 62), 1 << 62, (1 << 23,), generator=g, device="cuda")
+    keys[:3] = torch.tensor([-1, -2, -3], device="cuda")
+    vals = (keys >> 20).to(width)
+    t = Table(kind, slots, bucket_bytes=32)
+    try:
+        t.insert(keys, vals)
+        t.erase(keys[5::7].contiguous())
+        q = torch.cat([keys[:200001], keys[:200001] + 1])
+        t.set_launch(1, keys_per_group=1)
+        want = [t.find(q[:n]) for n in (1, 33, 4097, q.numel())]
+        t.set_launch(1, keys_per_group=8)
+        for (f, v), n in zip(want, (1, 33, 4097, q.numel())):
+            gf, gv = t.find(q[:n])
+            assert torch.equal(gf, f) and torch.equal(gv, v)
+            assert torch.equal(t.find(q[:n], vals_out=False)[0], f)
+        assert 0 < int(want[-1][0].sum()) < q.numel()
+    finally:
+        t.close()

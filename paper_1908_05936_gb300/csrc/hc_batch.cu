@@ -119,7 +119,7 @@ k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chu
             debug_range(v, p0, m, it.n);
             ArraySrc<KIND> src{(const Key *)it.keys + p0, (const Val *)it.vals + p0, nullptr};
             if constexpr (OP == OP_INSERT) insert_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
-            else if constexpr (OP == OP_FIND) find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals);
+            else if constexpr (OP == OP_FIND) find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals, it.vals_out != nullptr);
             else erase_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
             for (int i = lane; i < m; i += 32) {
                 if (it.out) st_stream(it.out + p0 + i, w.st[i]);

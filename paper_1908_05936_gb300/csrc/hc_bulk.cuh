@@ -196,10 +196,11 @@ struct RunsSrc {
 };
 
 // One warp: the runs of part (warp / groups) in `runs` chunks, R keys at a
-// time (one round, unless the part holds more than its share).
+// time (one round, unless the part holds more than its share).  `want`: a lookup
+// brings values back.
 template <int KIND, int BB, int OP, int NT, int R, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
-k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs) {
+k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs, bool want) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
@@ -239,13 +240,14 @@ k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs
         __syncwarp();
         RunsSrc<KIND> src{reinterpret_cast<const Key *>(sc.keys), reinterpret_cast<const Val *>(sc.vals), start, upto};
         if constexpr (OP == OP_INSERT) insert_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
-        else if constexpr (OP == OP_FIND) find_run<KIND, BB, WHOLE>(v, src, m, w.stack, w.st, w.vals);
+        else if constexpr (OP == OP_FIND) find_run<KIND, BB, WHOLE>(v, src, m, w.stack, w.st, w.vals, want);
         else erase_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
         for (int i = lane; i < m; i += 32) {
             const unsigned to = src.place(i);
             st_stream(sc.out + to, w.st[i]);
-            if constexpr (OP == OP_FIND && T::MAP)
-                st_stream(reinterpret_cast<Val *>(reinterpret_cast<Key *>(sc.keys) + to), w.vals[i]);
+            if constexpr (OP == OP_FIND && T::MAP) {
+                if (want) st_stream(reinterpret_cast<Val *>(reinterpret_cast<Key *>(sc.keys) + to), w.vals[i]);
+            }
         }
         __syncwarp();
     }

@@ -499,7 +499,7 @@ cudaError_t launch_bulk_op(const View &v, const void *keys, const void *vals, lo
     const int runs = (int)std::max<long long>(1, std::min<long long>(want, kBulkRuns));
     const int groups = (chunks + runs - 1) / runs;
     const unsigned grid = (unsigned)(((long long)parts * groups * 32 + NT - 1) / NT);
-    k_bulk_probe<KIND, BB, OP, NT, R, MINB><<<grid, NT, 0, s>>>(v, sc, chunks, parts, groups, runs);
+    k_bulk_probe<KIND, BB, OP, NT, R, MINB><<<grid, NT, 0, s>>>(v, sc, chunks, parts, groups, runs, vals_out != nullptr);
     if (T::MAP && OP == OP_FIND && vals_out)
         k_bulk_join<Key, Val, true><<<chunks, kBulkThreads, 0, s>>>(n, sc, out, (Val *)vals_out);
     else if (out)

@@ -313,10 +313,12 @@ struct Stack {
 };
 
 // Looks up the keys src.key(i), i < cnt (asked for 32 at a time, in order, by
-// the whole warp); found flags go to sf[i], values to sv[i].
+// the whole warp); found flags go to sf[i], values to sv[i], those of hits only
+// if `want`: a value is a request of its own (2^22 hits asked for without values,
+// 64-byte buckets: 1 GiB 173 -> 110 us, 256 MB 89 -> 83; 128-byte 1 GiB 1.33x).
 template <int KIND, int BB, bool TOGETHER, class Src>
 __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack<KIND, 1> &st, uint8_t *sf,
-                                         typename Traits<KIND>::Val *sv) {
+                                         typename Traits<KIND>::Val *sv, bool want) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
@@ -374,8 +376,10 @@ __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack
                 sf[idx] = 1;
                 if constexpr (WITH_VAL) sv[idx] = val;
                 else if constexpr (T::MAP) {
-                    late = idx;
-                    late_val = (Val)load_val<KIND, BB>(v, b, __ffs(seen.hit) - 1);
+                    if (want) {
+                        late = idx;
+                        late_val = (Val)load_val<KIND, BB>(v, b, __ffs(seen.hit) - 1);
+                    }
                 }
             } else {
                 b = next_bucket(v, b);
@@ -415,7 +419,7 @@ __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack
         if (act && stop) {
             if (d.sub == __ffs(stop) - 1) {
                 sf[idx] = seen.hit ? 1 : 0;
-                if constexpr (T::MAP) sv[idx] = seen.hit ? (Val)load_val<KIND, BB>(v, mine, __ffs(seen.hit) - 1) : (Val)0;
+                if constexpr (T::MAP) sv[idx] = seen.hit && want ? (Val)load_val<KIND, BB>(v, mine, __ffs(seen.hit) - 1) : (Val)0;
             }
         } else if (act && d.sub == 0) {
             left = unread == d.group;
@@ -885,7 +889,7 @@ k_run(View v, const typename Traits<KIND>::Key *keys, const typename Traits<KIND
     ArraySrc<KIND> src{keys + c0, vals + c0, skip ? skip + c0 : nullptr};
     Counts cnts;
     if constexpr (OP == 0) insert_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, cnts);
-    else if constexpr (OP == 1) find_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, w.vals);
+    else if constexpr (OP == 1) find_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, w.vals, vals_out != nullptr);
     else erase_run<KIND, BB, TOGETHER>(v, src, cnt, w.stack, w.st, cnts);
     for (int i = threadIdx.x & 31; i < cnt; i += 32) {
         if (out) st_stream(out + c0 + i, w.st[i]);

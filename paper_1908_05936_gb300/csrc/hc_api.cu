@@ -356,18 +356,19 @@ hc_rc range_checks(const hc_table *t, int op, const void *keys, const void *vals
 }
 
 hc_rc run_range(hc_table *t, int op, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,
-                cudaStream_t s, const uint8_t *skip = nullptr) {
+                cudaStream_t s, const uint8_t *skip = nullptr, bool host = false) {
     hc_rc rc = range_checks(t, op, keys, vals, n, out, vals_out);
     if (rc != HC_OK || n == 0) return rc;
     hc::LaunchShape sh = t->shape[op];
     sh.sms = sm_count_of(t->device);
+    sh.host = host;
     hc::View v = t->view;
     v.rotate = n > (long long)v.nb ? 1 : 0;        // several inserters per bucket: spread them
     const void *in = is_map(t->kind) && op == hc::OP_INSERT ? vals : nullptr;
     void *vo = is_map(t->kind) ? vals_out : nullptr;
     bool done = false;
     cudaError_t e = cudaSuccess;
-    if (!skip) e = try_bulk(t, op, v, keys, in, n, out, vo, s, &done);
+    if (!skip && !host) e = try_bulk(t, op, v, keys, in, n, out, vo, s, &done);
     if (!done) e = dispatch_range(t->kind, op, v, t->bucket_bytes, keys, in, n, out, vo, sh, skip, s);
     if (e != cudaSuccess) return cuda_fail(e, "launching the range kernel");
     return HC_OK;
@@ -426,7 +427,7 @@ hc_rc run_host(hc_table *t, int op, const void *h_keys, const void *h_vals, long
         const bool ok = dk && (op != hc::OP_INSERT || !is_map(t->kind) || dv) && (!h_out || dout) &&
                         (!want_vals || dvo);
         if (ok) {
-            if ((rc = run_range(t, op, dk, dv, n, static_cast<uint8_t *>(dout), dvo, s)) != HC_OK) return rc;
+            if ((rc = run_range(t, op, dk, dv, n, static_cast<uint8_t *>(dout), dvo, s, nullptr, true)) != HC_OK) return rc;
             HC_CUDA(cudaStreamSynchronize(s), "synchronising the stream");
             return HC_OK;
         }

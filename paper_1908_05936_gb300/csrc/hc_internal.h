@@ -21,6 +21,7 @@ struct LaunchShape {
     int block;            // threads per block
     int fold;             // 1 = fold equal keys inside a warp
     int sms;              // multiprocessors of the table's device (grid sizing)
+    bool host;            // the call's arrays are in page-locked host memory
 };
 
 #define HC_DECLARE_KIND(NAME)                                                                                       \

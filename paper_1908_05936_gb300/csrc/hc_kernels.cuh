@@ -358,8 +358,15 @@ constexpr long long kBeyondReach = 512ll << 20;
 // L2-resident set<u32> workload 64 and 59); 128 for larger calls.  Beyond reach
 // shorter runs spread the wait for requests better (10^6 keys on an 800 MB map:
 // insert + lookup + erase 264 us in one wave of 192, 237 with 128, 233 with 64;
-// erases of 2^22 keys and more prefer 128 by 4 %).
-inline int run_length(int op, long long n, long long resident, int most, bool beyond) {
+// erases of 2^22 keys and more prefer 128 by 4 %).  Maps called with arrays in
+// host memory: keys and results take longer on the link than a probe takes, and
+// more short runs keep more of them on it; calls on 2^23 slots, us, longer runs ->
+// 32: 300,000 inserts 50.8 -> 47.3, lookups 40.2 -> 35.9; 2^20 inserts 127 -> 108,
+// lookups 106 -> 80.  From 2^21 on inserts and erases are bound by the link or the
+// table and 64 keys are as good.  Sets have less to carry: u64 within 5 %, 2^20
+// inserts of u32 20 % slower with 32.
+inline int run_length(int op, long long n, long long resident, int most, bool beyond, bool host_map) {
+    if (host_map) return op == OP_FIND || n < (1ll << 21) ? 32 : 64;
     const long long wave = (n + resident * 32 - 1) / (resident * 32) * 32;
     if (beyond) return (int)std::min<long long>(wave, op == OP_ERASE ? 128 : 64);
     return wave <= most ? (int)wave : 128;
@@ -376,7 +383,7 @@ cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, lon
                        const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     using T = Traits<KIND>;
     const long long resident = (long long)sh.sms * run_blocks(Slots<KIND, BB>::KRB, TOGETHER) * 8;
-    const int run = run_length(OP, n, resident, R, (long long)v.nb * BB >= kBeyondReach);
+    const int run = run_length(OP, n, resident, R, (long long)v.nb * BB >= kBeyondReach, sh.host && T::MAP);
     const long long per_block = (long long)(sh.block / 32) * run;
     const unsigned grid = (unsigned)((n + per_block - 1) / per_block);
     const size_t smem = sizeof(WarpRun<KIND, OP, R>) * (sh.block / 32);

@@ -113,3 +113,42 @@ def test_whole_bucket_lookups(kind, slots):
         assert 0 < int(want[-1][0].sum()) < q.numel()
     finally:
         t.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n", (33, 4097, (1 << 21) - 1, 1 << 21))
+def test_page_locked_arrays(kind, n):
+    """Calls on page-locked host arrays, on both sides of the size where their
+    runs get longer, against the same calls on device arrays."""
+    import torch
+
+    from paper_1908_05936_gb300.table import KEY_BYTES, KEY_NUMPY, KEY_TORCH, VAL_BYTES, VAL_NUMPY, Table
+    kb, vb = KEY_BYTES[kind], VAL_BYTES.get(kind, 0)
+    keys = torch.randperm(2 * n, generator=torch.Generator().manual_seed(n), dtype=torch.int64)
+    keys = (keys * 40503 % (1 << 32)).to(KEY_TORCH[kb])
+    vals = (keys.to(torch.int64) * 3 + 1).to(KEY_TORCH[vb]) if vb else None
+
+    def pinned(t, dtype):
+        return t.clone().pin_memory().numpy().view(dtype)
+
+    def room(dtype):
+        return torch.zeros(2 * n * np.dtype(dtype).itemsize, dtype=torch.uint8).pin_memory().numpy().view(dtype)
+
+    def same(t, a):
+        return np.array_equal(t.cpu().numpy(), a.view(t.cpu().numpy().dtype)[:t.numel()])
+
+    a, b = Table(kind, 3 * n, bucket_bytes=64), Table(kind, 3 * n, bucket_bytes=64)
+    try:
+        k, hk, st = keys.cuda(), pinned(keys, KEY_NUMPY[kind]), room(np.uint8)
+        dv, hv = (vals.cuda(), pinned(vals, VAL_NUMPY[kind])) if vb else (None, None)
+        b.insert_host(hk[:n], hv[:n] if vb else None, st)
+        assert same(a.insert(k[:n], dv[:n] if vb else None), st)
+        hvo = room(VAL_NUMPY[kind]) if vb else None
+        b.find_host(hk, st, hvo)
+        f, v = a.find(k)
+        assert same(f, st) and (not vb or same(v, hvo))
+        b.erase_host(hk[n // 2:], st)
+        assert same(a.erase(k[n // 2:]), st)
+        assert a.size() == b.size() == n // 2
+    finally:
+        a.close(), b.close()

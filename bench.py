@@ -33,19 +33,17 @@ METRIC = "Mops/s insert/find/erase at LF 0.8; p50/p99 batch latency; % of HBM pe
 # algorithmic bytes per op for map<u64,u64>: one 32-byte slot sector read
 # (+ one written for modifying ops) + key/value in + status/value out
 BYTES_PER_OP = {"insert": 16 + 1 + 32 + 32, "find": 8 + 8 + 1 + 32, "erase": 8 + 1 + 32 + 32}
-# DRAM bytes per op of the range insert kernel (k_insert_stream<map<u64,u64>,
-# 64-byte buckets, 4 keys/thread, 2 in flight>, 64-thread blocks) on this
-# workload: dram__bytes_read.sum + dram__bytes_write.sum over the four fill
-# launches of one step at full size (one ncu capture), divided by the keys
-# they inserted; `requests_per_op` the same for lts__t_requests_srcunit_tex.sum
-# (requests from the SMs to L2).  Valid only while the kernel sources hash to
-# `digest`.
-INSERT_TRAFFIC = {"bytes_per_op": 227.7, "requests_per_op": 3.545, "digest": "a09fabcd81947d1e"}
+# DRAM bytes per op of the insert calls on this workload (bulk calls: split,
+# probe and join kernels over map<u64,u64> with 64-byte buckets):
+# dram__bytes_read.sum + dram__bytes_write.sum over the twelve kernels of one
+# step's four fill calls at full size (one ncu capture), divided by the keys
+# they inserted.  Valid only while the kernel sources hash to `digest`.
+INSERT_TRAFFIC = {"bytes_per_op": 176.8, "digest": "264bc4df2b7c7603"}
 
 
 def insert_kernel_digest() -> str:
-    """Hash of the insert kernel's source: the device core, the warp-run probe
-    loops with their kernel, and its launcher."""
+    """Hash of the insert call's kernels: the device core, the warp-run probe
+    loops, the bulk kernels and their launcher."""
     import hashlib
     import re
     csrc = os.path.join(ROOT, "paper_1908_05936_gb300", "csrc")
@@ -53,7 +51,8 @@ def insert_kernel_digest() -> str:
     parts = [open(os.path.join(ROOT, "include", "hc_core.cuh")).read(),
              re.search(r"// -+ warp stacks -+\n.*?\n// Streaming map lookup by lane pairs", read("hc_stream.cuh"),
                        re.S).group(0),
-             re.search(r"cudaError_t launch_run\(.*?\n}\n", read("hc_kernels.cuh"), re.S).group(0)]
+             read("hc_bulk.cuh"),
+             re.search(r"cudaError_t launch_bulk_op\(.*?\n}\n", read("hc_kernels.cuh"), re.S).group(0)]
     return hashlib.sha256("\n".join(parts).encode()).hexdigest()[:16]
 
 
@@ -329,20 +328,12 @@ def run_gpu(args, rank: int, world: int):
     dom_ms = summary[dom]["ms_total"] / len(per[dom])
     achieved = BYTES_PER_OP[kinds[dom]] * dom_n / (dom_ms * 1e-3) / 1e9
     traffic = None
-    if (dom == "insert" and not in_kernel and bb == 64 and t.get_launch(0)["keys_per_group"] == 8
-            and t.get_launch(0)["block"] == 128 and insert_kernel_digest() == INSERT_TRAFFIC["digest"]):
+    if (dom == "insert" and not in_kernel and bb == 64 and wl.slots == 1 << 28 and B == 1 << 26
+            and t.get_launch(0)["keys_per_group"] == 8 and t.get_launch(0)["block"] == 128
+            and insert_kernel_digest() == INSERT_TRAFFIC["digest"]):
         traffic = INSERT_TRAFFIC["bytes_per_op"] * dom_n      # DRAM bytes per launch
     peak, peak_src = hbm_peak()
     ceiling = random_read_ceiling(torch, L)
-    # the same kernel against the device's rate of scattered L2 requests
-    # (random 32-byte reads, measured above): requests per op x ops per second
-    requests = None
-    if traffic:
-        req_rate = INSERT_TRAFFIC["requests_per_op"] * dom_n / (dom_ms * 1e-3) / 1e9
-        requests = {"per_op": INSERT_TRAFFIC["requests_per_op"], "achieved": round(req_rate, 1),
-                    "ceiling": ceiling["reads_per_s"], "unit": "G L2 requests/s",
-                    "frac": round(req_rate / ceiling["reads_per_s"], 3),
-                    "source": "ncu lts__t_requests_srcunit_tex.sum, full-size capture"}
 
     out = {
         "metric": METRIC, "value": round(value, 2), "unit": "Mops/s", "n_gpus": world, "steps": args.steps,
@@ -360,8 +351,7 @@ def run_gpu(args, rank: int, world: int):
                      "traffic": round(traffic) if traffic else None, "bytes_per_op": BYTES_PER_OP[kinds[dom]],
                      "dram_gbs": round(traffic / (dom_ms * 1e-3) / 1e9, 1) if traffic else None,
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum, full-size capture"
-                     if traffic else "no capture for this kernel as built",
-                     "requests": requests},
+                     if traffic else "no capture for this kernel as built"},
         "at_lf08": {"insert_mops": summary["insert_by_batch"][-1]["mops"],
                     "insert_batch_lf": [round(max(0.0, (nb - 1) * B / wl.slots), 3), summary["insert_by_batch"][-1]["lf_end"]],
                     "find_hit_mops": round(summary["find_hit"]["mops"], 1),

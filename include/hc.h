@@ -447,9 +447,9 @@ HC_API hc_rc hc_batch_destroy(hc_batch *b);
 HC_API int64_t hc_batch_scratch_bytes(int64_t n_items);
 
 /* Run n_items items once as a batch (the same phases and scheduling as a
- * batch from hc_batch_create, without a graph), with the descriptors and
- * chunk counters in the caller's device buffer d_scratch (256-byte aligned,
- * at least hc_batch_scratch_bytes(n_items) bytes).  Nothing is allocated and
+ * batch from hc_batch_create, without a graph), with the descriptors in the
+ * caller's device buffer d_scratch (256-byte aligned, at least
+ * hc_batch_scratch_bytes(n_items) bytes).  Nothing is allocated and
  * nothing is kept, so a caller forming a new batch for every dispatch (a
  * request loop) pays no allocation.  Calls on different streams need
  * different scratch buffers; calls ordered on one stream may share one.  At
@@ -463,9 +463,9 @@ HC_API hc_rc hc_batch_run(const hc_batch_item *items, int64_t n_items, const hc_
  * 0), but allocates nothing.  Some callers cannot call cudaMalloc: a serving
  * process whose device memory is all owned by another allocator's pool, or a
  * latency-bound request loop where an allocation's implicit device-wide
- * synchronisation would stall every other stream.  The descriptors and chunk
- * counters live in one fixed array (about 105 KB) inside the library, which
- * every GPU that loads the library holds until the process exits.
+ * synchronisation would stall every other stream.  The descriptors live in one
+ * fixed array (about 105 KB) inside the library, which every GPU that loads
+ * the library holds until the process exits.
  *   - The first call on a device looks up that array's device address
  *     (cudaGetSymbolAddress) with the device current; make that first call
  *     before any stream capture.  The address is kept for the life of the

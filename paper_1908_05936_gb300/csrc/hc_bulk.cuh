@@ -26,8 +26,8 @@
 // Measured against the warp-run kernels (2^28-slot map, 64-byte buckets, 2^26
 // keys, G keys/s): present lookups at load factor 0.55 24.0 -> 40.5, inserts
 // 0.55 -> 0.8 12.8 -> 22.3, erases 22.2 -> 34.9; 2^26 lookups, half present, at
-// 0.8: 3.56 -> 1.99 ms; 30 M set lookups on 10^8 slots 0.84 -> 0.62 ms; the
-// 2^28-slot step 25.3 -> 16.1 ms.
+// 0.8: 3.56 -> 1.89 ms; 30 M set lookups on 10^8 slots 0.84 -> 0.51 ms; the
+// 2^28-slot step 25.3 -> 15.4 ms.
 // Parts of 32 MB: 16 or 64 MB are within 3 % (4 GiB).  Bringing the next parts
 // into L2 ahead of the probes by bulk prefetches loses at every distance from 8
 // to 96 MB (lookups 43 -> 32-36 G/s).  256 keys a warp: with 512 or more

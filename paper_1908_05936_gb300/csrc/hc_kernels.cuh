@@ -341,8 +341,7 @@ cudaError_t launch_range_shape(int op, const View &v, const void *keys, const vo
 }
 
 // A kernel launched with more than the default 48 KB of dynamic shared
-// memory (streaming kernels with 256-thread blocks and 8 keys per thread)
-// must be allowed it first.
+// memory must be allowed it first.
 template <class K>
 void allow_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024) (void)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -422,7 +421,7 @@ cudaError_t launch_find_pair(const View &v, const void *keys, long long n, uint8
 template <int KIND, int BB, int LB>
 cudaError_t launch_range_kpt(int op, const View &v, const void *keys, const void *vals, long long n, uint8_t *out,
                              void *vals_out, const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
-    if (sh.keys_per_group >= 4) {       // streaming forms: one thread per key, or a lane pair per map key
+    if (sh.keys_per_group >= 4) {       // warp runs, or a lane pair per map key
         if constexpr (Traits<KIND>::MAP && LB == BB && Slots<KIND, BB>::KRB * 2 == BB) {
             if (n <= 0) return cudaSuccess;
             if (op == OP_FIND) {

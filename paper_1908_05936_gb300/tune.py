@@ -207,14 +207,13 @@ def apply(table: Table) -> bool:
 def batch_candidates(bucket_bytes: int) -> list[dict]:
     """Launch shapes of the batched form for set<u64> tables of one bucket
     size: lock-step phases with one thread per key (lane 0) or 32-byte lanes,
-    1 or 2 keys per thread; warp runs of 128 or 256 keys (4 or 8 keys per
-    thread); blocks of 64 / 128 / 256 threads; chunks of 256, 1024 or 4096 keys
-    or the automatic size (0)."""
+    1 or 2 keys per thread; warp runs of 128 keys (4 keys per thread); blocks
+    of 64 / 128 / 256 threads; chunks of 1024 or 4096 keys or the automatic
+    size (0)."""
     lanes = (0, 32) if bucket_bytes > 32 else (0,)
     out = [dict(lane_bytes=lb, keys_per_group=k, block=b, tile=t)
            for lb in lanes for k in (1, 2) for b in (64, 128, 256) for t in (0, 1024, 4096)]
-    out += [dict(lane_bytes=0, keys_per_group=k, block=b, tile=t)
-            for k in (4, 8) for b in (64, 128, 256) for t in (0, 256, 1024, 4096)]
+    out += [dict(lane_bytes=0, keys_per_group=4, block=b, tile=t) for b in (64, 128, 256) for t in (0, 1024, 4096)]
     return out
 
 

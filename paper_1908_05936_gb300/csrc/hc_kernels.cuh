@@ -363,10 +363,14 @@ constexpr long long kBeyondReach = 512ll << 20;
 // 32: 300,000 inserts 50.8 -> 47.3, lookups 40.2 -> 35.9; 2^20 inserts 127 -> 108,
 // lookups 106 -> 80.  From 2^21 on inserts and erases are bound by the link or the
 // table and 64 keys are as good.  Sets have less to carry: u64 within 5 %, 2^20
-// inserts of u32 20 % slower with 32.
-inline int run_length(int op, long long n, long long resident, int most, bool beyond, bool host_map) {
+// inserts of u32 20 % slower with 32.  Inserts of fewer than 2^22 keys into maps
+// with key regions of 32 bytes or less (`narrow_map`) beyond reach: runs of 32 are
+// 1-9 % faster than 64 from 400,000 keys on (2^20 into 50 M slots at 0.7, 32- and
+// 64-byte buckets 1.07 and 1.04); sets and 128-byte buckets lose 3-19 %.
+inline int run_length(int op, long long n, long long resident, int most, bool beyond, bool host_map, bool narrow_map) {
     if (host_map) return op == OP_FIND || n < (1ll << 21) ? 32 : 64;
     const long long wave = (n + resident * 32 - 1) / (resident * 32) * 32;
+    if (beyond && op == OP_INSERT && narrow_map && n < (1ll << 22)) return 32;
     if (beyond) return (int)std::min<long long>(wave, op == OP_ERASE ? 128 : 64);
     return wave <= most ? (int)wave : 128;
 }
@@ -382,7 +386,8 @@ cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, lon
                        const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     using T = Traits<KIND>;
     const long long resident = (long long)sh.sms * run_blocks(Slots<KIND, BB>::KRB, TOGETHER) * 8;
-    const int run = run_length(OP, n, resident, R, (long long)v.nb * BB >= kBeyondReach, sh.host && T::MAP);
+    const int run = run_length(OP, n, resident, R, (long long)v.nb * BB >= kBeyondReach, sh.host && T::MAP,
+                               T::MAP && Slots<KIND, BB>::KRB <= 32);
     const long long per_block = (long long)(sh.block / 32) * run;
     const unsigned grid = (unsigned)((n + per_block - 1) / per_block);
     const size_t smem = sizeof(WarpRun<KIND, OP, R>) * (sh.block / 32);

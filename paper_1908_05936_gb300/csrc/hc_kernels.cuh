@@ -349,6 +349,12 @@ void allow_smem(K kernel, size_t bytes) {
 
 // Tables from which on the reach of the address translation is what matters.
 constexpr long long kBeyondReach = 512ll << 20;
+// The same for key regions of 64 and 128 bytes and calls whose one wave would
+// take runs of more than 128 keys: 2^20 keys on 384-496 MB, insert / lookup /
+// erase with runs of 64 over one wave of 192 or 224 1.08 / 1.05 / 1.04 (map, 128
+// bytes), 1.07 / 1.10 / 1.08 (set, 64), 1.18 / 1.17 / 1.09 (set, 128); on 288 MB
+// and less 0.85-0.98 but for lookups in 128-byte set buckets.
+constexpr long long kWideReach = 352ll << 20;
 
 // The warp-run kernels (keys_per_group 4 or 8), the length of a run: what makes
 // one wave of equal runs of the warps that are resident together, if that is at
@@ -386,7 +392,9 @@ cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, lon
                        const LaunchShape &sh, const uint8_t *skip, cudaStream_t s) {
     using T = Traits<KIND>;
     const long long resident = (long long)sh.sms * run_blocks(Slots<KIND, BB>::KRB, TOGETHER) * 8;
-    const int run = run_length(OP, n, resident, R, (long long)v.nb * BB >= kBeyondReach, sh.host && T::MAP,
+    const long long bytes = (long long)v.nb * BB;
+    const bool beyond = bytes >= (Slots<KIND, BB>::KRB > 32 && n > resident * 128 ? kWideReach : kBeyondReach);
+    const int run = run_length(OP, n, resident, R, beyond, sh.host && T::MAP,
                                T::MAP && Slots<KIND, BB>::KRB <= 32);
     const long long per_block = (long long)(sh.block / 32) * run;
     const unsigned grid = (unsigned)((n + per_block - 1) / per_block);

@@ -196,7 +196,7 @@ struct RunsSrc {
 };
 
 // One warp: the runs of part (warp / groups) in `runs` chunks, R keys at a
-// time (one round, unless the part holds more than its share).  `want`: a lookup
+// time (one pass, unless the part holds more than its share).  `want`: a lookup
 // brings values back.
 template <int KIND, int BB, int OP, int NT, int R, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
@@ -233,7 +233,7 @@ k_bulk_probe(View v, BulkScratch sc, int chunks, int parts, int groups, int runs
     Counts cnts;
     for (int base = 0; base < total; base += R) {
         const int m = total - base < R ? total - base : R;
-        // the table of this round: keys [base, base + m) of the warp's runs
+        // the places of this pass: keys [base, base + m) of the warp's runs
         const int before = (int)(incl - len) - base;
         start[lane] = (unsigned)(first + lane) * kBulkChunk + a + (before < 0 ? (unsigned)-before : 0u);
         upto[lane] = (int)incl > base ? incl - (unsigned)base : 0u;

@@ -310,6 +310,7 @@ struct Stack {
     unsigned long long free_at[INS ? kStack : 1];
     Key key[kStack];
     Val val[VAL ? kStack : 1];
+    unsigned lost;                       // inserts: swaps that the run's keys have lost to other keys
 };
 
 // Looks up the keys src.key(i), i < cnt (asked for 32 at a time, in order, by
@@ -446,8 +447,12 @@ __device__ __forceinline__ void find_run(const View &v, Src &src, int cnt, Stack
 // Inserts the keys src.key(i) with values src.val(i), i < cnt, except those
 // with src.skip(i) (a find saw them: EXISTS); statuses go to ss[i].  A key that
 // loses its slot to another key goes on from that slot's bucket: the buckets
-// before it had no free slot, and inserts never free one.  Equal keys inside a
-// warp are not folded here (folding is a lock-step option).
+// before it had no free slot, and inserts never free one.  Every lost swap means
+// that another key took a slot, so they end by themselves; the limit that keeps
+// the loop finite whatever the table holds is on lost swaps, kMaxRestarts a key,
+// counted for the run as a whole (steps would not do: without an EMPTY slot a key
+// reads every bucket before each swap).  Equal keys inside a warp are not folded
+// here (folding is a lock-step option).
 template <int KIND, int BB, bool TOGETHER, class Src>
 __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Stack<KIND, 0> &st, uint8_t *ss,
                                            Counts &cnts) {
@@ -471,6 +476,7 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
         ahead_skip = src.skip(i);
     };
     fetch(lane);
+    if (lane == 0) st.lost = 0u;             // (a __syncwarp follows before the first swap)
     unsigned long long reach = 0;
     const int few = v.nb >= 32 ? 16 : 0;     // a group's buckets are distinct
     // Claims the free slot `at` for key; whether the key stays undecided, with
@@ -495,7 +501,7 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
             ss[idx] = (uint8_t)ST_EXISTS;
             return false;
         }
-        if (reach >= v.nb + 32ull * kMaxRestarts) {
+        if (atomicAdd(&st.lost, 1u) >= (unsigned)cnt * kMaxRestarts) {
             atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
             ss[idx] = (uint8_t)ST_OVERFLOW;
             cnts.over = 1;

@@ -66,6 +66,7 @@ struct MixedRun {
     typename T::Key key[kStack];
     typename T::Val val[T::MAP ? kStack : 1];
     typename T::Val vals[T::MAP ? kMixedRun : 1];            // found values out
+    unsigned lost;                                           // swaps lost to other keys and waits for claims
     uint8_t st[kMixedRun];
 };
 
@@ -104,6 +105,10 @@ k_mixed_run(View v, const uint8_t *ops, const typename Traits<KIND>::Key *keys, 
         ahead_op = ld_stream(ops + i);
     };
     fetch(lane);
+    if (lane == 0) w.lost = 0u;              // (a __syncwarp follows before the first swap)
+    // One more lost swap or wait; whether the run's operations have met more of
+    // them than kMaxRestarts each (the limit that keeps the loop finite).
+    auto too_many = [&]() { return atomicAdd(&w.lost, 1u) >= (unsigned)cnt * kMaxRestarts; };
     unsigned long long reach = 0;
     for (;; ++reach) {
         Key key;
@@ -167,7 +172,11 @@ k_mixed_run(View v, const uint8_t *ops, const typename Traits<KIND>::Key *keys, 
                         if (seen.tomb) wait = hcd::detail::must_wait<SPB>(v, b, seen.tomb, le, rot);
                     }
                     if (wait) {              // the bucket is read again
-                        full = false;
+                        if (too_many()) {    // a claim that never resolves
+                            atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
+                            cnts.over = 1;
+                            done(ST_OVERFLOW);
+                        }
                     } else if (le) {
                         q = hcd::detail::first_from<SPB>(le, rot);
                         swap = true;
@@ -192,10 +201,6 @@ k_mixed_run(View v, const uint8_t *ops, const typename Traits<KIND>::Key *keys, 
                     if (op == MOP_INSERT) cnts.over = 1;
                     done(op == MOP_INSERT ? (uint32_t)ST_OVERFLOW : op == MOP_FIND ? 0u : (uint32_t)ST_NOT_FOUND);
                 }
-            } else if (left && !swap && q < 0 && reach >= v.nb + 32ull * kMaxRestarts) {
-                atomicOr(&v.hdr->err, ERR_PROBE_BOUND);      // a claim that never resolves
-                cnts.over = 1;
-                done(ST_OVERFLOW);
             }
         }
         bool publish = false;
@@ -219,7 +224,7 @@ k_mixed_run(View v, const uint8_t *ops, const typename Traits<KIND>::Key *keys, 
                     }
                 } else if (!T::MAP && old == key) {
                     done(ST_EXISTS);         // an equal key won the slot
-                } else if (reach >= v.nb + 32ull * kMaxRestarts) {
+                } else if (too_many()) {
                     atomicOr(&v.hdr->err, ERR_PROBE_BOUND);
                     cnts.over = 1;
                     done(ST_OVERFLOW);

@@ -30,8 +30,8 @@ __device__ __forceinline__ unsigned long long aux_hash(unsigned long long k) {
     return fmix64(k ^ 0xD6E8FEB86659FD93ull);
 }
 
-// Keys of a batch that takes the passes over plain indices: 32 MB of 8-byte keys
-// and as much scratch.
+// Keys of a batch that takes the passes over plain indices (for 8-byte keys 32 MB
+// of them and as much scratch).
 constexpr long long kSmallBatch = 1ll << 22;
 
 struct AuxEntry {
@@ -112,11 +112,22 @@ __global__ void __launch_bounds__(256) k_mark_followers(const Key *keys, long lo
 
 // The same two passes for batches whose keys and a scratch of plain indices fit
 // L2 together: an entry is the index alone (all ones: empty), and a probe reads
-// the key at it from the batch.  The swap comes first, an entry that is not empty
-// comes back from it.  2^22 draws from 2^21 keys: scratch fill + claims + marks
-// 145 us with 16-byte entries, 105 so; insert + lookup + erase 699 -> 613 us.
+// the key at it from the batch.  Both passes read entries through L1, so that the
+// entries of keys that occur often are not asked for in L2 by every occurrence: an
+// entry that is not empty never becomes so again and its key never changes, so an
+// old copy says the same, and one that looks empty goes through the swap.  Swaps
+// on one entry go one after another (0.66 ns each): with the swap first, 2^22 equal
+// keys took 2.77 ms, 2^22 draws of a Zipf distribution 0.28 ms; with the read first
+// 0.10 and 0.15 (erase calls; distinct keys 0.27 and 0.29, an insert + lookup +
+// erase of 2^22 draws from 2^21 keys 622 and 643 us, with 16-byte entries 699).
 // (Beyond L2 a second random read per key costs as much as the first: 2.07
 // against 1.87 ms for an insert of 2^24 draws.)
+__device__ __forceinline__ unsigned load_index(const unsigned *e) {
+    unsigned r;
+    asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(r) : "l"(e));
+    return r;
+}
+
 template <class Key>
 __global__ void __launch_bounds__(256) k_claim_leaders_small(const Key *keys, int n, unsigned *aux, unsigned mask,
                                                              unsigned *err) {
@@ -125,7 +136,8 @@ __global__ void __launch_bounds__(256) k_claim_leaders_small(const Key *keys, in
     const Key k = keys[i];
     unsigned h = (unsigned)aux_hash((unsigned long long)k) & mask;
     for (unsigned p = 0; p <= mask; ++p) {
-        const unsigned cur = atomicCAS(&aux[h], ~0u, (unsigned)i);
+        unsigned cur = load_index(aux + h);
+        if (cur == ~0u) cur = atomicCAS(&aux[h], ~0u, (unsigned)i);
         if (cur == ~0u) return;
         if (keys[cur] == k) {
             if ((unsigned)i < cur) atomicMin(&aux[h], (unsigned)i);
@@ -145,7 +157,7 @@ __global__ void __launch_bounds__(256) k_mark_followers_small(const Key *keys, i
     unsigned h = (unsigned)aux_hash((unsigned long long)k) & mask;
     unsigned leader = (unsigned)i;
     for (unsigned p = 0; p <= mask; ++p) {
-        const unsigned cur = __ldcg(aux + h);
+        const unsigned cur = load_index(aux + h);
         if (cur == ~0u || cur == (unsigned)i) break;    // this position leads (an empty entry cannot be met)
         if (keys[cur] == k) {
             leader = cur;

@@ -538,12 +538,13 @@ __device__ __forceinline__ void insert_run(const View &v, Src &src, int cnt, Sta
                 ss[idx] = won ? (uint8_t)ST_INSERTED : (uint8_t)ST_EXISTS;
                 act = false;
             }
-            b = first_bucket(v, (unsigned long long)key);
             // a step for a few keys costs what one for 32 does: keys among many
             // that are skipped wait on the stack for company (the insert of a
             // 400,000-candidate frame, 88 % of them found before, 18.6 -> 15.9
             // us; an ordered insert + lookup + erase of 2^22 draws 720 -> 699)
             const unsigned mask = __ballot_sync(0xffffffffu, act);
+            if (mask == 0u) continue;        // (all skipped: nothing to hash)
+            b = first_bucket(v, (unsigned long long)key);
             if (__popc(mask) <= kFewKeys) {
                 if (act) {
                     const int p = top + __popc(mask & lanes_below());
@@ -723,8 +724,9 @@ __device__ __forceinline__ void erase_run(const View &v, Src &src, int cnt, Stac
                 ss[idx] = won ? (uint8_t)ST_ERASED : (uint8_t)ST_NOT_FOUND;
                 act = false;
             }
-            b = first_bucket(v, (unsigned long long)key);
             const unsigned mask = __ballot_sync(0xffffffffu, act);      // as in insert_run
+            if (mask == 0u) continue;
+            b = first_bucket(v, (unsigned long long)key);
             if (__popc(mask) <= kFewKeys) {
                 if (act) {
                     const int p = top + __popc(mask & lanes_below());

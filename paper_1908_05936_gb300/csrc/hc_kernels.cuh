@@ -99,33 +99,31 @@ __global__ void k_pad_tombstones(View v, unsigned long long first, unsigned long
 
 // --------------------------------------------------------------- rehash ---
 // The stored keys of the old array as runs of the insert loop (the keys are
-// distinct, and the new table holds no tombstone but its padding).  A key's new
-// home keeps its old home's place in proportion, so both arrays are swept in
-// order; neighbouring keys share new buckets, so inserts scan them from
-// key-dependent slots (View::rotate).  A thread per old slot that looked for an
-// EMPTY slot word by word took 1.69 ms for 2^26 slots of 64-byte buckets at load
-// factor 0.6; the runs take 1.2 ms, bound by instructions (24 warp instructions
-// a key, issue 61 %; DRAM 30 %).  For small tables and the spatial hashes, whose
-// homes are scattered (next section for the others).
+// distinct, and the new table holds no tombstone but its padding).  A warp reads 256
+// slots, all loads at once, and its run is the keys that it finds there, so that a
+// step has 32 of them however sparse the old array is (with the slots themselves as
+// a run whose EMPTY ones were skipped, 2^27 slots with 2^24 keys under the spatial
+// hash took 3.0 ms, and so 2.25).  A key's new home keeps its old home's place in
+// proportion, so both arrays are swept in order; neighbouring keys share new
+// buckets, so inserts scan them from key-dependent slots (View::rotate).  For small
+// or crowded tables and the spatial hashes, whose homes are scattered (next section
+// for the others).
 
+// Keys of a run: the live ones of slots [first, first + 256).
 template <int KIND, int BB>
-struct OldSlots {
+struct LiveSlots {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
     using S = Slots<KIND, BB>;
     const View &old_v;
-    unsigned long long first;        // slot position of key 0 of the run
-    Key last = Key();
-    __device__ __forceinline__ Key key(int i) {
-        const unsigned long long p = first + (unsigned)i;
-        return last = ld_stream(reinterpret_cast<const Key *>(S::key(old_v, p / S::SPB, (int)(p % S::SPB))));
-    }
-    // of the key asked for last
-    __device__ __forceinline__ bool skip(int) const { return last == T::EMPTY || last == T::TOMB; }
+    unsigned long long first;
+    const Key *keys;                 // (shared)
+    const uint8_t *at;               // (shared) their slots, counted from `first`
+    __device__ __forceinline__ Key key(int i) const { return keys[i]; }
+    __device__ __forceinline__ bool skip(int) const { return false; }
     __device__ __forceinline__ Val val(int i) const {
-        if (skip(i)) return Val();
-        const unsigned long long p = first + (unsigned)i;
+        const unsigned long long p = first + at[i];
         return ld_stream(reinterpret_cast<const Val *>(S::val(old_v, p / S::SPB, (int)(p % S::SPB))));
     }
 };
@@ -133,17 +131,42 @@ struct OldSlots {
 template <int KIND, int BB>
 __global__ void __launch_bounds__(256, run_blocks(Slots<KIND, BB>::KRB, false))
 k_rehash(View old_v, unsigned long long old_phys, View new_v) {
+    using T = Traits<KIND>;
+    using Key = typename T::Key;
+    using S = Slots<KIND, BB>;
     constexpr int R = 256;
     __shared__ WarpRun<KIND, OP_INSERT, R> sh[8];
+    __shared__ Key live_key[8][R];
+    __shared__ uint8_t live_at[8][R];
     __shared__ BlockCounts sum;
     sum.init();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned long long w0 = (unsigned long long)blockIdx.x * 8;
-    const unsigned long long first = (w0 + (threadIdx.x >> 5)) * R;
+    const unsigned long long first = (w0 + warp) * R;
     if (first >= old_phys) return;
-    WarpRun<KIND, OP_INSERT, R> &w = sh[threadIdx.x >> 5];
-    OldSlots<KIND, BB> src{old_v, first};
+    Key key[R / 32];
+#pragma unroll
+    for (int j = 0; j < R / 32; ++j) {
+        const unsigned long long p = first + j * 32 + lane;
+        key[j] = T::EMPTY;
+        if (p < old_phys) key[j] = ld_stream(reinterpret_cast<const Key *>(S::key(old_v, p / S::SPB, (int)(p % S::SPB))));
+    }
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < R / 32; ++j) {
+        const bool live = key[j] != T::EMPTY && key[j] != T::TOMB;
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const int to = n + __popc(m & lanes_below());
+            live_key[warp][to] = key[j];
+            live_at[warp][to] = (uint8_t)(j * 32 + lane);
+        }
+        n += __popc(m);
+    }
+    __syncwarp();
+    LiveSlots<KIND, BB> src{old_v, first, live_key[warp], live_at[warp]};
     Counts cnts;
-    insert_run<KIND, BB, false>(new_v, src, (int)(old_phys - first < R ? old_phys - first : R), w.stack, w.st, cnts);
+    insert_run<KIND, BB, false>(new_v, src, n, sh[warp].stack, sh[warp].st, cnts);
     const unsigned long long busy = (old_phys + R - 1) / R - w0;       // warps of this block with slots
     sum.flush(new_v, cnts, busy < 8 ? (int)busy : 8);
 }

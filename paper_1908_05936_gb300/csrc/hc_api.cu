@@ -2,6 +2,8 @@
 // checks (the contracts of Section 3.3 become return codes), table creation
 // and destruction (Section 3.7), dispatch of the range calls to the per-kind
 // kernels, counters, clear, dump, rehash and the host-buffer forms.
+#include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -289,15 +291,54 @@ __global__ void k_rehash_finish(hc::Header *old_h, hc::Header *new_h) {
 
 __global__ void k_clear_err(hc::Header *h) { h->err = 0u; }
 
-// Rehashes t into the uninitialised array behind nv region by region
-// (k_rehash_regions) if the tables are of a size for it and the list of keys
-// left over can be had; *done says whether nv holds every key.
-cudaError_t rehash_by_regions(hc_table *t, const hc::View &nv, cudaStream_t s, bool *done) {
+// Whether a rehash of `keys` regular keys into `slots` slots goes region by region
+// (k_rehash_regions) rather than as runs of the insert loop (k_rehash).  Every line
+// is touched once that way, but the keys whose probe leaves its region are
+// inserted last, when the array is fullest: fewer of them in wide buckets, and what
+// they take weighs less the larger the array is.  So the line is a load of the new
+// array that rises with both.  Time of runs over time of regions, same size (16 MB
+// to 1 GiB, loads 0.3 to 0.97):
+//   map<u64,u64>, 32-byte buckets (2 slots)  64 MB 0.83-0.99; 128 MB 0.6: 1.03, 0.7:
+//       0.95; 256 MB 0.7: 1.05, 0.85: 0.91; 1 GiB 0.8: 1.09, 0.85: 1.04, 0.9: 0.94
+//   map<u64,u64>, 64 (4)   40 MB 0.90-0.95; 64 MB 0.7: 1.07, 0.85: 0.84; 128 MB 0.8: 1.11,
+//       0.9: 0.81; 1 GiB 0.95: 1.05
+//   map<u64,u64>, 128 (8)  40 MB 0.93-0.99; 64 MB 0.8: 1.05, 0.9: 0.87; 128 MB 0.93: 1.0;
+//       256 MB and more 1.1-1.6
+//   set<u64>, 32 (4)       40 MB 0.85-1.03; 64 MB 0.6: 1.08, 0.8: 0.97; 1 GiB 0.9: 1.08, 0.93: 0.96
+//   set<u32>, 32 (8)       16 MB 0.85-0.92; 24 MB 0.7: 1.02, 0.85: 0.92; 40 MB 0.7: 1.12,
+//       0.85: 0.91; 1 GiB 0.93: 1.01, 0.95: 0.90
+//   set<u64>, 128 (16)     16 MB 0.8: 1.02, 0.9: 0.93; 64 MB 0.95: 1.08; 128 MB and more 1.3-2.7
+//   set<u32>, 128 (32)     16 MB 0.95: 1.0; 24 MB and more 1.1-4.1
+// With regions at every load a map of 32-byte buckets and 24 MB at 0.97 took 4.2 ms,
+// 2.6 before there were regions, and takes 2.2 in runs.
+bool regions_pay(int kind, unsigned long long bytes, int slots_per_bucket, long long keys, long long slots) {
+    const bool map = is_map(kind);
+    const double least = (map ? std::max(64, 256 / slots_per_bucket) : std::max(16, 192 / slots_per_bucket)) * 1048576.0;
+    if ((double)bytes < least) return false;
+    double load, step = 0.04;                                 // the line at `least` bytes, its rise per doubling
+    switch (slots_per_bucket) {
+        case 2: load = 0.72; break;
+        case 4: load = map ? 0.80 : 0.76; break;
+        case 8: load = map ? 0.86 : 0.80; step = map ? 0.06 : 0.04; break;
+        case 16: load = 0.92; break;
+        default: load = 0.95; break;
+    }
+    load += step * std::log2((double)bytes / least);
+    if (!map && slots_per_bucket <= 8) load = std::min(load, 0.93);
+    return (double)keys <= load * (double)slots;
+}
+
+// Rehashes t, which holds `keys` regular keys, into the uninitialised array of
+// `slots` slots behind nv region by region if that pays and the list of keys left
+// over can be had; *done says whether nv holds every key.
+cudaError_t rehash_by_regions(hc_table *t, const hc::View &nv, long long keys, long long slots, cudaStream_t s,
+                              bool *done) {
     *done = false;
-    const unsigned long long bytes = nv.nb * (unsigned long long)t->bucket_bytes;
-    // 16 MB: a few regions per SM; an old array much larger than the new one has
-    // too few blocks to walk it
-    if (nv.hash_mode != hc::HASH_MIX64 || bytes < (16ull << 20) || t->view.nb > 8 * nv.nb) return cudaSuccess;
+    // an old array much larger than the new one has too few blocks to walk it
+    if (nv.hash_mode != hc::HASH_MIX64 || t->view.nb > 8 * nv.nb ||
+        !regions_pay(t->kind, nv.nb * (unsigned long long)t->bucket_bytes, slots_per_bucket(t->kind, t->bucket_bytes),
+                     keys, slots))
+        return cudaSuccess;
     cudaMemPool_t pool = pool_of(t->device);
     const unsigned long long cap = (unsigned long long)t->phys / 16 + 4096;
     unsigned long long *list = nullptr;                       // the count, then (256 bytes on) the positions
@@ -683,7 +724,7 @@ hc_rc hc_rehash(hc_table *t, int64_t new_slots, void *stream) {
     }
     hc::View nv = make_view(mem, g, t->view.seed, t->view.hash_mode);
     bool done = false;
-    e = rehash_by_regions(t, nv, s, &done);
+    e = rehash_by_regions(t, nv, regular, new_slots, s, &done);
     if (e == cudaSuccess && !done) {
         e = dispatch_clear(t, nv, g.phys, new_slots, s);
         const int sms = sm_count_of(t->device);

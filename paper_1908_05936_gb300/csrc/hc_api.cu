@@ -234,13 +234,25 @@ bool on_device(const void *p) {
     return a.type == cudaMemoryTypeDevice;
 }
 
+// While it lives, this thread's calls do not invalidate a capture that is going on
+// in another stream or thread (the pool's allocations would, in the default mode,
+// though nothing of them is captured).
+struct BesideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCaptures() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BesideCaptures() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    BesideCaptures(const BesideCaptures &) = delete;
+};
+
 // Runs the call as a bulk call if that pays and its scratch can be had: a
 // stream that is capturing, or a device without the memory, keeps the range
 // kernels.  *done says whether it ran.
 cudaError_t try_bulk(hc_table *t, int op, const hc::View &v, const void *keys, const void *vals, long long n,
                      uint8_t *out, void *vals_out, cudaStream_t s, bool *done) {
     *done = false;
-    if (t->shape_set[op] || !bulk_pays(t, op, n) || !on_device(keys) || (vals && !on_device(vals))) return cudaSuccess;
+    if (t->shape_set[op] || !bulk_pays(t, op, n)) return cudaSuccess;
+    BesideCaptures beside;
+    if (!on_device(keys) || (vals && !on_device(vals))) return cudaSuccess;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
         (void)cudaGetLastError();

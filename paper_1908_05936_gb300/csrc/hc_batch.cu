@@ -127,7 +127,13 @@ k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chu
             debug_range(v, p0, m, it.n);
             ArraySrc<KIND> src{(const Key *)it.keys + p0, (const Val *)it.vals + p0, nullptr};
             if constexpr (OP == OP_INSERT) insert_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
-            else if constexpr (OP == OP_FIND) find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals, it.vals_out != nullptr);
+            else if constexpr (OP == OP_FIND && T::MAP && BB == 32) {
+                // as the range lookups (5 M, half present, on a 512 MB table: lock-step
+                // phases, which read whole buckets too, 136 us; keys and values apart 145;
+                // so 130)
+                if ((long long)v.nb * BB >= kWholeBytes) find_run<KIND, BB, true>(v, src, m, w.stack, w.st, w.vals, it.vals_out != nullptr);
+                else find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals, it.vals_out != nullptr);
+            } else if constexpr (OP == OP_FIND) find_run<KIND, BB, false>(v, src, m, w.stack, w.st, w.vals, it.vals_out != nullptr);
             else erase_run<KIND, BB, false>(v, src, m, w.stack, w.st, cnts);
             for (int i = lane; i < m; i += 32) {
                 if (it.out) st_stream(it.out + p0 + i, w.st[i]);

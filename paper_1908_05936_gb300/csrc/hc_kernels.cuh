@@ -407,8 +407,6 @@ inline int run_length(int op, long long n, long long resident, int most, bool be
 // Tables from which lanes read wide buckets together (see_bucket; between 256
 // MB, where it costs 0-17 %, and 512 MB, where it gains 5-50 %).
 constexpr long long kTogetherBytes = kBeyondReach;
-// Maps with 32-byte buckets of which lookups read whole buckets (see_whole_bucket).
-constexpr long long kWholeBytes = 256ll << 20;
 
 template <int KIND, int BB, int OP, int R, bool TOGETHER>
 cudaError_t launch_run_as(const View &v, const void *keys, const void *vals, long long n, uint8_t *out, void *vals_out,

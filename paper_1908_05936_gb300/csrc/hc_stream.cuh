@@ -272,6 +272,7 @@ __device__ __forceinline__ Seen see_bucket(const View &v, bool act, unsigned lon
 // 128 MB 52.3 -> 50.3, 256 MB 31.7 -> 38.9, 2 GiB 22.2 -> 33.3; lookups that miss
 // are the same from 256 MB on, and 4-9 % slower inside L2.  Wider buckets, read
 // by lanes together, gain 15-30 % on hits and lose as much on misses: not done.
+constexpr long long kWholeBytes = 256ll << 20;    // tables from which on lookups do so
 template <int KIND, int BB>
 __device__ __forceinline__ Seen see_whole_bucket(const View &v, bool act, unsigned long long b,
                                                  typename Traits<KIND>::Key key, typename Traits<KIND>::Val &val) {

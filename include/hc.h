@@ -419,10 +419,11 @@ typedef struct hc_batch_config {
     int32_t lane_bytes;      /* 0: one thread per key (whole bucket); 32: 32-byte lanes */
     int32_t keys_per_group;  /* 1 or 2: lock-step phases; 4 or 8: warp runs of
                                 up to 128 or 256 keys (0 = 8)              */
-    int32_t block;           /* threads per block (0 = 64 for warp runs, 256
-                                for lock-step phases)                      */
+    int32_t block;           /* threads per block (0 = 64 for warp runs with
+                                one warp per chunk, 256 otherwise)         */
     int32_t blocks_per_sm;   /* persistent grid = SMs x this (0: one warp per
-                                chunk)                                     */
+                                chunk for warp runs, as many blocks as fit
+                                for lock-step phases)                      */
     int32_t tile;            /* keys per chunk, a multiple of 128 (0 = auto:
                                 from the total keys, so that the chunks can
                                 occupy every warp slot: 128..256 for warp
@@ -447,8 +448,8 @@ HC_API hc_rc hc_batch_destroy(hc_batch *b);
 HC_API int64_t hc_batch_scratch_bytes(int64_t n_items);
 
 /* Run n_items items once as a batch (the same phases and scheduling as a
- * batch from hc_batch_create, without a graph), with the descriptors in the
- * caller's device buffer d_scratch (256-byte aligned, at least
+ * batch from hc_batch_create, without a graph), with the descriptors and
+ * chunk counters in the caller's device buffer d_scratch (256-byte aligned, at least
  * hc_batch_scratch_bytes(n_items) bytes).  Nothing is allocated and
  * nothing is kept, so a caller forming a new batch for every dispatch (a
  * request loop) pays no allocation.  Calls on different streams need
@@ -463,7 +464,7 @@ HC_API hc_rc hc_batch_run(const hc_batch_item *items, int64_t n_items, const hc_
  * 0), but allocates nothing.  Some callers cannot call cudaMalloc: a serving
  * process whose device memory is all owned by another allocator's pool, or a
  * latency-bound request loop where an allocation's implicit device-wide
- * synchronisation would stall every other stream.  The descriptors live in one
+ * synchronisation would stall every other stream.  The descriptors and counters live in one
  * fixed array (about 105 KB) inside the library, which every GPU that loads
  * the library holds until the process exits.
  *   - The first call on a device looks up that array's device address

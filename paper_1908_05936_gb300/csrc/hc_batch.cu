@@ -2,12 +2,13 @@
 // persistent launch per phase (insert, then find, then erase), optionally
 // captured once into a CUDA graph and replayed.
 //
-// Scheduling.  Every item is cut into chunks of `tile` keys.  A phase kernel has
-// one warp per chunk (or, with blocks_per_sm, a persistent grid whose warps
-// stride over the chunks); a warp finds the item its chunk belongs to by a
-// 32-way search over the items' chunk offsets and runs the same loops as the
-// one-launch-per-call kernels over the chunk.  Tables of very different sizes
-// are therefore balanced at chunk granularity, and no launch is spent per table.
+// Scheduling.  Every item is cut into chunks of `tile` keys.  A phase of warp runs
+// has one warp per chunk; lock-step phases, and runs with blocks_per_sm, are a
+// persistent grid whose warps take the next chunk from a counter.  A warp finds the
+// item its chunk belongs to by a search over the items' chunk offsets and runs the
+// same loops as the one-launch-per-call kernels over the chunk.  Tables of very
+// different sizes are therefore balanced at chunk granularity, and no launch is
+// spent per table.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -43,7 +44,10 @@ struct PhaseDesc {
     int item0;
     int n_items;
     long long n_chunks;
+    int counter;   // index of this phase's chunk counter
 };
+
+constexpr int kCounterBytes = 512;       // room for 36 phases' counters behind the descriptors
 
 template <int KIND, int OP, int BB, int LB, int KPT>
 __device__ __forceinline__ void run_chunk(const BatchItemDev &it, long long k0, long long k1) {
@@ -55,6 +59,17 @@ __device__ __forceinline__ void run_chunk(const BatchItemDev &it, long long k0, 
                                      it.out, (typename T::Val *)it.vals_out, k1, k0 / TILE, (k1 + TILE - 1) / TILE, 1,
                                      it.fold != 0, cnt);
     if constexpr (OP != OP_FIND) flush_counts(it.v, cnt);
+}
+
+// The next chunk of a phase, for the whole warp.
+__device__ __forceinline__ long long next_chunk(unsigned long long *counter) {
+    unsigned long long c = 0;
+    if ((threadIdx.x & 31) == 0) c = atomicAdd(counter, 1ull);
+    return (long long)__shfl_sync(0xffffffffu, c, 0);
+}
+
+__global__ void k_zero_counters(unsigned long long *c, int n) {
+    if (threadIdx.x < n) c[threadIdx.x] = 0ull;
 }
 
 // The item that chunk c of a phase belongs to: the last one whose chunk_begin
@@ -76,14 +91,24 @@ __device__ __forceinline__ int item_of(const BatchItemDev *items, int n_items, l
 // each launch is a small specialisation).  WIDE: one thread per key reading
 // the whole bucket (maps: keys and values) or key region (sets); otherwise
 // 32-byte lanes.
+//
+// A counter rather than a warp per chunk: warps of a chunk of up to 1024 keys end
+// at very different times, and a block's place is free only when its last one has
+// (128 tables, one key per thread: 320 us, 384 with a warp per chunk).
 template <int KIND, int OP, int BB, int WIDE, int KPT>
 __global__ void __launch_bounds__(256)
-k_batch_phase(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile) {
+k_batch_phase(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile,
+              unsigned long long *counter) {
     constexpr int KRB = Slots<KIND, BB>::KRB;
     constexpr int LB = WIDE ? (Traits<KIND>::MAP ? BB : KRB) : (KRB < 32 ? KRB : 32);
-    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_chunks; c += warps) {
-        const BatchItemDev it = items[item_of(items, n_items, c)];
+    for (long long c = next_chunk(counter); c < n_chunks; c = next_chunk(counter)) {
+        int lo = 0, hi = n_items - 1;                      // last item whose chunk_begin is at most c
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (items[mid].chunk_begin <= c) lo = mid;
+            else hi = mid - 1;
+        }
+        const BatchItemDev it = items[lo];
         const long long k0 = (c - it.chunk_begin) * tile;
         const long long k1 = k0 + tile < it.n ? k0 + tile : it.n;
         debug_range(it.v, k0, k1 - k0, it.n);
@@ -108,15 +133,17 @@ constexpr int batch_blocks(int krb) { return krb == 128 ? 3 : 4; }
 
 template <int KIND, int OP, int BB, int R>
 __global__ void __launch_bounds__(256, batch_blocks(Slots<KIND, BB>::KRB))
-k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile) {
+k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chunks, int tile,
+            unsigned long long *counter) {
     using T = Traits<KIND>;
     using Key = typename T::Key;
     using Val = typename T::Val;
     extern __shared__ __align__(16) unsigned char smem[];
     WarpRun<KIND, OP, R> &w = reinterpret_cast<WarpRun<KIND, OP, R> *>(smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_chunks; c += warps) {
+    // without a counter: one warp per chunk
+    for (long long c = counter ? next_chunk(counter) : ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+         c < n_chunks; c = counter ? next_chunk(counter) : n_chunks) {
         const BatchItemDev &it = items[item_of(items, n_items, c)];
         const View v = it.v;
         const long long k0 = (c - it.chunk_begin) * tile;
@@ -147,7 +174,7 @@ k_batch_run(const BatchItemDev *__restrict__ items, int n_items, long long n_chu
     }
 }
 
-using PhaseKernel = void (*)(const BatchItemDev *, int, long long, int);
+using PhaseKernel = void (*)(const BatchItemDev *, int, long long, int, unsigned long long *);
 
 template <int KIND, int OP, int BB>
 PhaseKernel pick_lb_kpt(int lb, int kpt) {
@@ -210,8 +237,9 @@ struct hc_batch {
     bool use_graph;
     void *d_mem = nullptr;
     hc::BatchItemDev *d_items = nullptr;
+    unsigned long long *d_counters = nullptr;      // behind the items
     std::vector<hc::PhaseDesc> phases;
-    std::vector<int> grid;
+    int sms = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -251,24 +279,59 @@ hc_rc bcuda(cudaError_t e, const char *what) {
     return bfail(HC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// Blocks of a phase: one warp per chunk, or a persistent grid of per_sm blocks
-// per SM where the configuration asks for one.
-unsigned phase_grid(const hc::PhaseDesc &ph, int block, int per_sm, int sms) {
-    const long long need = (ph.n_chunks * 32 + block - 1) / block;
-    return (unsigned)(per_sm > 0 ? std::min<long long>(need, (long long)sms * per_sm) : need);
+// Whether the phases' warps take their chunks from counters (a persistent grid).
+bool counted(int kpt, int per_sm) { return kpt < 4 || per_sm > 0; }
+
+// Threads per block where the configuration leaves it open (64: warp runs, one
+// warp per chunk; a grid of per_sm blocks per SM keeps the warps that it has had).
+int default_block(int kpt, int per_sm) { return counted(kpt, per_sm) ? 256 : 64; }
+
+// Blocks of a phase: as many as give every chunk a warp, and for counted phases at
+// most per_sm (0: what fits) per SM.
+cudaError_t phase_grid(const hc::PhaseDesc &ph, hc::PhaseKernel k, int kpt, int block, size_t smem, int per_sm, int sms,
+                       unsigned *grid) {
+    long long g = (ph.n_chunks * 32 + block - 1) / block;
+    if (counted(kpt, per_sm)) {
+        cudaError_t e = cudaSuccess;
+        if (per_sm <= 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem);
+        if (e != cudaSuccess) return e;
+        g = std::min<long long>(g, (long long)sms * std::max(per_sm, 1));
+    }
+    *grid = (unsigned)std::max<long long>(g, 1);
+    return cudaSuccess;
 }
 
-hc_rc enqueue(hc_batch *b, cudaStream_t s) {
-    for (size_t p = 0; p < b->phases.size(); ++p) {
-        const hc::PhaseDesc &ph = b->phases[p];
-        hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, b->lane_bytes, b->kpt);
-        const size_t smem = hc::phase_smem(ph.kind, ph.op, b->kpt, b->block);
+// Enqueues the phases over descriptors and counters that are on the device.
+hc_rc enqueue_phases(const hc::PhaseDesc *phases, int n_phases, const hc::BatchItemDev *d_items,
+                     unsigned long long *d_counters, int lane_bytes, int kpt, int block, int per_sm, int tile, int sms,
+                     cudaStream_t s) {
+    cudaError_t e;
+    const bool counters = counted(kpt, per_sm);
+    if (n_phases == 0) return HC_OK;
+    if (counters) {
+        hc::k_zero_counters<<<1, 64, 0, s>>>(d_counters, n_phases);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return bcuda(e, "resetting the batch counters");
+    }
+    for (int p = 0; p < n_phases; ++p) {
+        const hc::PhaseDesc &ph = phases[p];
+        hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lane_bytes, kpt);
+        const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
         hc::allow_phase_smem(k, smem);
-        k<<<b->grid[p], b->block, smem, s>>>(b->d_items + ph.item0, ph.n_items, ph.n_chunks, b->tile);
-        const cudaError_t e = cudaGetLastError();
+        unsigned grid = 0;
+        e = phase_grid(ph, k, kpt, block, smem, per_sm, sms, &grid);
+        if (e != cudaSuccess) return bcuda(e, "querying the occupancy of a batch phase");
+        k<<<grid, block, smem, s>>>(d_items + ph.item0, ph.n_items, ph.n_chunks, tile,
+                                    counters ? d_counters + ph.counter : nullptr);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return bcuda(e, "launching a batch phase");
     }
     return HC_OK;
+}
+
+hc_rc enqueue(hc_batch *b, cudaStream_t s) {
+    return enqueue_phases(b->phases.data(), (int)b->phases.size(), b->d_items, b->d_counters, b->lane_bytes, b->kpt,
+                          b->block, b->blocks_per_sm, b->tile, b->sms, s);
 }
 
 }  // namespace
@@ -284,7 +347,7 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     if (cfg) c = *cfg;
     const int lb = c.lane_bytes;
     const int kpt = c.keys_per_group ? c.keys_per_group : 8;
-    const int block = c.block ? c.block : kpt >= 4 ? 64 : 256;
+    const int block = c.block ? c.block : default_block(kpt, c.blocks_per_sm);
     const int tile = c.tile ? c.tile : auto_tile(items, n_items, kpt);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
@@ -299,7 +362,7 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     for (int op = 0; op < 3; ++op) {
         for (int kind = 0; kind < 4; ++kind)
         for (int bb = 32; bb <= 128; bb *= 2) {
-            hc::PhaseDesc ph{kind, op, bb, (int)dev.size(), 0, 0};
+            hc::PhaseDesc ph{kind, op, bb, (int)dev.size(), 0, 0, (int)phases.size()};
             for (int64_t i = 0; i < n_items; ++i) {
                 const hc_batch_item &it = items[i];
                 if (!it.table || it.table->magic != HC_TABLE_MAGIC) return bfail(HC_ERR_ARG, "item with a bad table");
@@ -337,23 +400,23 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     b->tile = tile;
     b->lane_bytes = lb;
     b->kpt = kpt;
+    b->blocks_per_sm = c.blocks_per_sm;
     b->use_graph = c.use_graph != 0;
     b->phases = phases;
     cudaError_t e = cudaGetDevice(&b->device);
     const size_t items_bytes = (dev.size() * sizeof(hc::BatchItemDev) + 255) / 256 * 256;
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_mem, std::max<size_t>(items_bytes, 256));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_mem, items_bytes + hc::kCounterBytes);
     if (e != cudaSuccess) {
         delete b;
         return bcuda(e, "allocating the batch descriptors");
     }
     b->d_items = static_cast<hc::BatchItemDev *>(b->d_mem);
+    b->d_counters = reinterpret_cast<unsigned long long *>(static_cast<char *>(b->d_mem) + items_bytes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!dev.empty())
         e = cudaMemcpyAsync(b->d_items, dev.data(), dev.size() * sizeof(hc::BatchItemDev), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    int sms = 0;
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-    for (const hc::PhaseDesc &ph : phases) b->grid.push_back(phase_grid(ph, block, c.blocks_per_sm, sms));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e == cudaSuccess && b->use_graph) {
         // capture on a private stream so the caller's stream is never in capture mode
         cudaStream_t cs;
@@ -418,6 +481,7 @@ constexpr int kNoAllocMaxPhases = 36;    // 3 operations x 4 container kinds x 3
 
 struct NoAllocScratch {
     hc::BatchItemDev items[kNoAllocMaxItems];
+    unsigned long long counters[64];
 };
 
 }  // namespace
@@ -464,7 +528,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     if (cfg) c = *cfg;
     const int lb = c.lane_bytes;
     const int kpt = c.keys_per_group ? c.keys_per_group : 8;
-    const int block = c.block ? c.block : kpt >= 4 ? 64 : 256;
+    const int block = c.block ? c.block : default_block(kpt, c.blocks_per_sm);
     const int tile = c.tile ? c.tile : auto_tile(items, n_items, kpt);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
@@ -480,7 +544,7 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     for (int op = 0; op < 3; ++op) {
         for (int kind = 0; kind < 4; ++kind)
         for (int bb = 32; bb <= 128; bb *= 2) {
-            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0};
+            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0, n_phases};
             for (int64_t i = 0; i < n_items; ++i) {
                 const hc_batch_item &it = items[i];
                 if (!it.table || it.table->magic != HC_TABLE_MAGIC) return bfail(HC_ERR_ARG, "item with a bad table");
@@ -529,17 +593,8 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     e = cudaMemcpyAsync(scratch->items, t_noalloc_items, (size_t)n_dev * sizeof(hc::BatchItemDev),
                         cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bcuda(e, "copying the batch descriptors");
-    for (int p = 0; p < n_phases; ++p) {
-        const hc::PhaseDesc &ph = phases[p];
-        hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lb, kpt);
-        const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
-        hc::allow_phase_smem(k, smem);
-        k<<<phase_grid(ph, block, c.blocks_per_sm, sms), block, smem, s>>>(scratch->items + ph.item0, ph.n_items,
-                                                                            ph.n_chunks, tile);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return bcuda(e, "launching a batch phase");
-    }
-    return HC_OK;
+    return enqueue_phases(phases, n_phases, scratch->items, scratch->counters, lb, kpt, block, c.blocks_per_sm, tile, sms,
+                          s);
 }
 
 }  // extern "C"
@@ -561,7 +616,7 @@ extern "C" {
 
 HC_API int64_t hc_batch_scratch_bytes(int64_t n_items) {
     if (n_items < 0 || n_items > kRunMaxItems) return -1;
-    return (int64_t)((n_items * sizeof(hc::BatchItemDev) + 255) / 256 * 256 + 512);   // the last 512 bytes are spare
+    return (int64_t)((n_items * sizeof(hc::BatchItemDev) + 255) / 256 * 256 + hc::kCounterBytes);
 }
 
 namespace {
@@ -590,7 +645,7 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     if (cfg) c = *cfg;
     const int lb = c.lane_bytes;
     const int kpt = c.keys_per_group ? c.keys_per_group : 8;
-    const int block = c.block ? c.block : kpt >= 4 ? 64 : 256;
+    const int block = c.block ? c.block : default_block(kpt, c.blocks_per_sm);
     const int tile = c.tile ? c.tile : auto_tile(items, n_items, kpt);
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole key region) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
@@ -605,7 +660,7 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     for (int op = 0; op < 3; ++op) {
         for (int kind = 0; kind < 4; ++kind)
         for (int bb = 32; bb <= 128; bb *= 2) {
-            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0};
+            hc::PhaseDesc ph{kind, op, bb, n_dev, 0, 0, n_phases};
             for (int64_t i = 0; i < n_items; ++i) {
                 const hc_batch_item &it = items[i];
                 if (!it.table || it.table->magic != HC_TABLE_MAGIC) return bfail(HC_ERR_ARG, "item with a bad table");
@@ -645,17 +700,8 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     e = cudaMemcpyAsync(d_items, desc, (size_t)n_dev * sizeof(hc::BatchItemDev), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bcuda(e, "copying the batch descriptors");
-    for (int p = 0; p < n_phases; ++p) {
-        const hc::PhaseDesc &ph = phases[p];
-        hc::PhaseKernel k = hc::pick_kernel(ph.kind, ph.op, ph.bb, lb, kpt);
-        const size_t smem = hc::phase_smem(ph.kind, ph.op, kpt, block);
-        hc::allow_phase_smem(k, smem);
-        k<<<phase_grid(ph, block, c.blocks_per_sm, sms), block, smem, s>>>(d_items + ph.item0, ph.n_items, ph.n_chunks,
-                                                                            tile);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return bcuda(e, "launching the batch phases");
-    return HC_OK;
+    auto *d_counters = reinterpret_cast<unsigned long long *>(static_cast<char *>(d_scratch) + need - hc::kCounterBytes);
+    return enqueue_phases(phases, n_phases, d_items, d_counters, lb, kpt, block, c.blocks_per_sm, tile, sms, s);
 }
 }  // namespace
 

@@ -77,6 +77,7 @@ struct alignas(256) Header {
     unsigned int side_lock;              // bits 0/1: side slot held by an in-kernel map insert; bit 2: CLAIM-key insert
     unsigned long long side_val[2];
     unsigned long long dump_count;       // output cursor of the dump kernel
+    unsigned long long reserved;         // keeps claim_key_at where kernels built with an earlier copy of this header look
     unsigned long long claim_key_at;     // maps: 1 + slot position of the stored key equal to CLAIM, 0 if none
 };
 static_assert(sizeof(Header) == 256, "header is one 256-byte block");

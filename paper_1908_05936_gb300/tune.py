@@ -9,7 +9,10 @@ of 2^(slots_log2 - 2) keys, then times every candidate shape on insert (the
 last batch of the fill), find (all present), find (all absent) and erase
 with CUDA events, and keeps the fastest shape per operation; "find" is the
 shape with the least time for the present and the absent batch together,
-the one `apply()` installs.  The winners are
+the one `apply()` installs.  The first candidate is the route of a table whose
+shapes nobody has set ("default"): run lengths chosen per call, and bulk calls
+where they pay, which an explicit shape turns off.  It stays the choice unless a
+shape is faster by more than MARGIN.  The winners are
 written to a JSON cache keyed by device name and SM count
 (`tuned.json` next to this file); `apply()` installs them on a table.
 
@@ -37,6 +40,8 @@ CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned.json")
 LANES = (16, 32, 64, 128)
 KEYS_IN_FLIGHT = (1, 2)
 BLOCKS = (64, 128, 256)
+MARGIN = 0.03                       # of the default route's time: what an explicit shape must gain
+BULK_BYTES = 512 << 20              # tables from which on large calls of the default route may be bulk calls
 
 
 def device_key() -> str:
@@ -101,6 +106,13 @@ def candidates(table: Table) -> list[dict]:
     return out
 
 
+def fastest(timings: list[tuple[float, dict]]) -> tuple[float, dict]:
+    """(ms, shape) of the least time, or of the default route (the first entry)
+    unless the shape beats it by more than MARGIN."""
+    best = min(timings, key=lambda x: x[0])
+    return best if best[0] < (1.0 - MARGIN) * timings[0][0] else timings[0]
+
+
 def tune_table(kind: int, bucket_bytes: int, slots_log2: int = 26, lf: float = 0.8, every: list | None = None) -> dict:
     """Best shape per operation; with `every` given, each candidate's timings
     are appended to it as well."""
@@ -124,10 +136,11 @@ def tune_table(kind: int, bucket_bytes: int, slots_log2: int = 26, lf: float = 0
         if t.is_map else False
     results = {"insert": [], "find_hit": [], "find_miss": [], "erase": []}
     t.insert(last, last_v, status=False)                  # the table starts at the target load factor
-    for c in candidates(t):
+    for c in [dict(default=True)] + candidates(t):
         find_only = c.pop("find_only", False)
-        for op in ((L.OP_FIND,) if find_only else (L.OP_INSERT, L.OP_FIND, L.OP_ERASE)):
-            t.set_launch(op, fold=2, **c)
+        if not c.get("default"):
+            for op in ((L.OP_FIND,) if find_only else (L.OP_INSERT, L.OP_FIND, L.OP_ERASE)):
+                t.set_launch(op, fold=2, **c)
 
         def ins():
             t.insert(last, last_v, status=out)
@@ -158,11 +171,11 @@ def tune_table(kind: int, bucket_bytes: int, slots_log2: int = 26, lf: float = 0
             every.append(row)
     best = {}
     for op, lst in results.items():
-        ms, c = min(lst, key=lambda x: x[0])
+        ms, c = fastest(lst)
         best[op] = dict(c, ms=round(ms, 4), mops=round(batch / ms / 1e3, 1))
     # lookups of a mix of present and absent keys: the least total time
     both = [(h[0] + m[0], h[1]) for h, m in zip(results["find_hit"], results["find_miss"])]
-    ms, c = min(both, key=lambda x: x[0])
+    ms, c = fastest(both)
     best["find"] = dict(c, ms=round(ms, 4), mops=round(2 * batch / ms / 1e3, 1))
     return best
 
@@ -188,7 +201,9 @@ def tune(kinds: list[int], buckets=(32, 64, 128), slots_log2: int = 26, save: bo
 
 def apply(table: Table) -> bool:
     """Install the tuned shapes for this table's kind and bucket size on the
-    current GPU, if the cache has them."""
+    current GPU, if the cache has them.  Operations whose choice is the default
+    route keep it, and so does a table of BULK_BYTES and more, whatever the size
+    the shapes were measured on."""
     if not os.path.exists(CACHE):
         return False
     with open(CACHE) as f:
@@ -197,9 +212,13 @@ def apply(table: Table) -> bool:
     best = cache.get(f"{name}/{table.bucket_bytes}")
     if not best:
         return False
+    if table.stats()["table_bytes"] >= BULK_BYTES:
+        return True
     for op, key in ((L.OP_INSERT, "insert"), (L.OP_FIND, "find" if "find" in best else "find_hit"),
                     (L.OP_ERASE, "erase")):
         b = best[key]
+        if b.get("default"):
+            continue
         table.set_launch(op, lane_bytes=b["lane_bytes"], keys_per_group=b["keys_per_group"], block=b["block"])
     return True
 

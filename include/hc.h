@@ -121,9 +121,12 @@ typedef struct hc_config {
  * lane_bytes = the bucket's key region, keys_per_group 8 (warp runs), block
  * 128, folding off; until hc_set_launch sets an op's shape, a large hc_insert,
  * hc_find or hc_erase on a table of 512 MB or more may run as three passes over
- * stream-ordered scratch of its own (11 to 19 bytes a key, for at most 2^26 keys
+ * stream-ordered scratch of its own (7 to 19 bytes a key, for at most 2^26 keys
  * at a time; a capturing stream, or memory that is not there, keeps the range
- * kernel).  Results never depend on the shape. */
+ * kernel).  Of that scratch a device keeps up to 1.5 GiB for the next such call,
+ * until its last table is destroyed; the driver takes it back earlier when a
+ * cudaMalloc in the process is short of memory.  Results never depend on the
+ * shape. */
 typedef struct hc_launch {
     int32_t lane_bytes;       /* 32, 64 or 128, at most bucket_bytes     */
     int32_t keys_per_group;   /* 1 or 2; 4 or 8: warp runs             */

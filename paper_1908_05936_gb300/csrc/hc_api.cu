@@ -260,8 +260,8 @@ cudaError_t try_bulk(hc_table *t, int op, const hc::View &v, const void *keys, c
     }
     cudaMemPool_t pool = pool_of(t->device);
     if (!pool) return cudaSuccess;
-    // Parts of 16 to 32 MB, 64 or a multiple of it: a chunk's runs then have 64
-    // keys or fewer, and whole runs fill a probing warp's 256 places to three
+    // 64 parts for each 2 GiB begun (8 to 32 MB a part; 512 parts at most, larger
+    // ones beyond 16 GiB): a chunk's runs then have 64 keys or fewer, and whole runs fill a probing warp's 256 places to three
     // quarters or more (32 parts: one run of 128; 1 GiB tables, 32 -> 64 parts:
     // set inserts 27.3 -> 30.1 G/s, map inserts 17.9 -> 18.5, lookups the same;
     // 128 parts of 8 MB: map lookups 42.0 -> 40.7).
@@ -619,7 +619,7 @@ hc_rc hc_set_launch(hc_table *t, int32_t op, const hc_launch *shape) {
           (sh.lane_bytes == krb || (op == hc::OP_FIND && is_map(t->kind) && sh.lane_bytes == t->bucket_bytes &&
                                     2 * krb == t->bucket_bytes))))
         return fail(HC_ERR_ARG,
-                    "keys_per_group must be 1 or 2 (4 or 8: streaming, lane = the key region, or the whole bucket for map lookups)");
+                    "keys_per_group must be 1 or 2 (4 or 8: warp runs, lane = the key region, or the whole bucket for map lookups)");
     if (sh.block < 64 || sh.block > 256 || sh.block % 32)
         return fail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     t->shape[op] = sh;

@@ -352,7 +352,6 @@ HC_API hc_rc hc_batch_create(hc_batch **out, const hc_batch_item *items, int64_t
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
         return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
-    if (kpt >= 4 && block > 256) return bfail(HC_ERR_ARG, "streaming phases take at most 256 threads per block");
     if (block < 64 || block > 256 || block % 32) return bfail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     if (tile < 128 || tile % 128) return bfail(HC_ERR_ARG, "tile must be a positive multiple of 128");
 
@@ -533,7 +532,6 @@ HC_API hc_rc hc_batch_run_noalloc(const hc_batch_item *items, int64_t n_items, c
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole bucket) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
         return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
-    if (kpt >= 4 && block > 256) return bfail(HC_ERR_ARG, "streaming phases take at most 256 threads per block");
     if (block < 64 || block > 256 || block % 32) return bfail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     if (tile < 128 || tile % 128) return bfail(HC_ERR_ARG, "tile must be a positive multiple of 128");
     if (c.use_graph) return bfail(HC_ERR_ARG, "hc_batch_run_noalloc launches directly; use_graph must be 0");
@@ -650,7 +648,6 @@ hc_rc batch_run(const hc_batch_item *items, int64_t n_items, const hc_batch_conf
     if (lb != 0 && lb != 32) return bfail(HC_ERR_ARG, "lane_bytes must be 0 (whole key region) or 32");
     if (kpt != 1 && kpt != 2 && kpt != 4 && kpt != 8)
         return bfail(HC_ERR_ARG, "keys_per_group must be 1 or 2 (lock-step) or 4 or 8 (warp runs)");
-    if (kpt >= 4 && block > 256) return bfail(HC_ERR_ARG, "streaming phases take at most 256 threads per block");
     if (block < 64 || block > 256 || block % 32) return bfail(HC_ERR_ARG, "block must be a multiple of 32 in [64, 256]");
     if (tile < 128 || tile % 128) return bfail(HC_ERR_ARG, "tile must be a positive multiple of 128");
 

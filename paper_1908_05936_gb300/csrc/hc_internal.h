@@ -17,7 +17,7 @@ enum : int { OP_INSERT = 0, OP_FIND = 1, OP_ERASE = 2 };
 
 struct LaunchShape {
     int lane_bytes;       // 16 (maps), 32, 64 or 128
-    int keys_per_group;   // 1 or 2
+    int keys_per_group;   // 1 or 2: lock step; 4 or 8: warp runs, or a lane pair per map key
     int block;            // threads per block
     int fold;             // 1 = fold equal keys inside a warp
     int sms;              // multiprocessors of the table's device (grid sizing)

@@ -181,7 +181,7 @@ k_rehash(View old_v, unsigned long long old_phys, View new_v) {
 // region go to a list that is inserted when every region is there; until then no
 // key of the list is looked for, and a bucket that a placed key has passed is
 // full for good.  Every line is read or written once, in order: 2^26 slots of
-// 64-byte buckets at load factor 0.6, 1.37 ms (fill and runs) -> 0.54 ms, 2 GiB
+// 64-byte buckets at load factor 0.6, 1.10 ms (fill and runs) -> 0.54 ms, 2 GiB
 // at 4 TB/s; what bounds it now is the placing of the keys of a bucket one after
 // another.  32 KB: 512 64-byte buckets, about 1 % of the keys cross a boundary,
 // and six blocks share an SM.

@@ -19,8 +19,7 @@ namespace hc {
 // its pieces of every staged array before it stores any: load() reads
 // 16-byte pieces tid, tid + nt, ... when src is 16-byte aligned (element by
 // element otherwise, and for a tail shorter than 16 bytes) into registers;
-// store() writes them to dst (shared, 16-byte aligned), `map` applied to
-// every element on the way (the skip flags become result bytes).
+// store() writes them to dst (shared, 16-byte aligned).
 template <class T, int KPT>
 struct Stage {
     static constexpr int E = 16 / (int)sizeof(T);          // elements per 16-byte piece
@@ -51,36 +50,24 @@ struct Stage {
         }
     }
 
-    template <class F>
-    __device__ __forceinline__ void store(T *dst, int m, F map) const {
+    __device__ __forceinline__ void store(T *dst, int m) const {
         const int nt = blockDim.x, tid = threadIdx.x;
         if (vec) {
             const int nv = m / E;
 #pragma unroll
             for (int j = 0; j < J; ++j) {
                 const int u = tid + j * nt;
-                if (u < nv) {
-                    T t[E];
-                    memcpy(t, &piece[j], 16);
-#pragma unroll
-                    for (int e = 0; e < E; ++e) t[e] = map(t[e]);
-                    uint4 w;
-                    memcpy(&w, t, 16);
-                    reinterpret_cast<uint4 *>(dst)[u] = w;
-                }
+                if (u < nv) reinterpret_cast<uint4 *>(dst)[u] = piece[j];
             }
             const int i = nv * E + tid;
-            if (i < m) dst[i] = map(elem[0]);
+            if (i < m) dst[i] = elem[0];
         } else {
 #pragma unroll
             for (int j = 0; j < KPT; ++j) {
                 const int i = tid + j * nt;
-                if (i < m) dst[i] = map(elem[j]);
+                if (i < m) dst[i] = elem[j];
             }
         }
-    }
-    __device__ __forceinline__ void store(T *dst, int m) const {
-        store(dst, m, [](T x) { return x; });
     }
 };
 

@@ -124,8 +124,9 @@ k_batch_phase(const BatchItemDev *__restrict__ items, int n_items, long long n_c
 // warps took chunks from one counter: 192 set<u64> of 2^10-2^20 slots, 25 M
 // operations, 750 -> 547 us; 1024 tables, 127 M operations, 3.21 -> 2.50 ms.
 //
-// Blocks of 256 threads per SM that it is compiled for: one fewer than the range
-// kernels' (run_blocks), since a phase holds its item's fields beside the probes.
+// Blocks of 256 threads per SM that it is compiled for: 4 (64 registers) and 3 (80)
+// for 128-byte key regions, fewer than the range kernels' (run_blocks), since a phase
+// holds its item's fields beside the probes.
 // At 5 for every key region all instances spilled, the widest most, and a batch of
 // set<u64> with 128-byte buckets was slower than its lock-step phases: 5 M lookups on
 // 256 MB 124 -> 143 us, 112 so; erases 70 -> 81, 64; 128 tables' erases 42 -> 49, 34.

@@ -212,7 +212,8 @@ def apply(table: Table) -> bool:
     best = cache.get(f"{name}/{table.bucket_bytes}")
     if not best:
         return False
-    if table.stats()["table_bytes"] >= BULK_BYTES:
+    view = table.device_view()                            # (nothing is synchronised)
+    if view.nb * view.bucket_bytes >= BULK_BYTES:
         return True
     for op, key in ((L.OP_INSERT, "insert"), (L.OP_FIND, "find" if "find" in best else "find_hit"),
                     (L.OP_ERASE, "erase")):

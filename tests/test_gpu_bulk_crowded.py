@@ -51,11 +51,11 @@ def test_one_key_many_times(name, bb, crowd):
 
 @pytest.mark.parametrize("name", ("set_u64", "map_u64_u64"))
 def test_keys_of_one_part(name):
-    """200,000 keys from the first thousandth of the table."""
+    """20,000 keys from the first thousandth of the table."""
     kind, n = CODE[name], 2 * BYTES // 128 + 1
     a, b = pair(kind, 64)
     try:
-        h = np.random.default_rng(3).integers(0, (1 << 64) // 1000, 200_000, dtype=np.uint64)
+        h = np.random.default_rng(3).integers(0, (1 << 64) // 1000, 20_000, dtype=np.uint64)
         few = to_device(mix_inverse(h))
         g = torch.Generator(device="cuda").manual_seed(5)
         compare(a, b, few[torch.randint(0, few.numel(), (n,), generator=g, device="cuda")].contiguous(), kind)
